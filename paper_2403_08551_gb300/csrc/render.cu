@@ -55,6 +55,15 @@ struct RSmem {
     float* s_tgt;  // [3 * Cfg::kPix], 16-byte aligned
 };
 
+// Place of pixel p (row-major in the tile) in a partial image: with blocks of
+// several rows, odd blocks swap neighbouring rows (a multiple of 4 pixels
+// stays together).
+template <class Cfg>
+__device__ __forceinline__ int part_at(int p) {
+    if (Cfg::ROWS == 1 || Cfg::T != 16) return p;
+    return p ^ (((p / (Cfg::ROWS * Cfg::T)) & 1) * Cfg::T);
+}
+
 // Renders tile t (the block's threads together). `phase` is the staging
 // mbarrier's parity, carried from tile to tile by persistent blocks.
 template <class Cfg>
@@ -94,13 +103,23 @@ __device__ __forceinline__ void render_tile(int t, uint32_t& phase, const RSmem<
     // now (cp.async): their latency, long when the target is read from host
     // memory over the host link, overlaps the accumulation below.
     if (target) {
-        for (int p = threadIdx.x; p < NPIX; p += NT) {
-            const int x = x0 + p % T, y = y0 + p / T;
-            if (x < d.W && y < d.H) {
-                const float* src = target + 3 * (d.pix_base + (int64_t)y * d.W + x);
-                cp_async4(&s_tgt[3 * p], src);
-                cp_async4(&s_tgt[3 * p + 1], src + 1);
-                cp_async4(&s_tgt[3 * p + 2], src + 2);
+        const float* t0 = target + 3 * (d.pix_base + (int64_t)y0 * d.W + x0);
+        const bool whole = x0 + T <= d.W && y0 + T <= d.H;
+        if (whole && d.W % 4 == 0 && (reinterpret_cast<uintptr_t>(t0) & 15) == 0) {
+            // whole tile, every row of it 16-byte aligned: 3 T / 4 copies a row
+            for (int q = threadIdx.x; q < 3 * NPIX / 4; q += NT) {
+                const int yy = q / (3 * T / 4), c = q % (3 * T / 4);
+                cp_async16(&s_tgt[4 * q], t0 + (int64_t)yy * 3 * d.W + 4 * c);
+            }
+        } else {
+            for (int p = threadIdx.x; p < NPIX; p += NT) {
+                const int x = x0 + p % T, y = y0 + p / T;
+                if (x < d.W && y < d.H) {
+                    const float* src = target + 3 * (d.pix_base + (int64_t)y * d.W + x);
+                    cp_async4(&s_tgt[3 * p], src);
+                    cp_async4(&s_tgt[3 * p + 1], src + 1);
+                    cp_async4(&s_tgt[3 * p + 2], src + 2);
+                }
             }
         }
     }
@@ -166,26 +185,42 @@ __device__ __forceinline__ void render_tile(int t, uint32_t& phase, const RSmem<
         __syncthreads();
     }
 
-    // Partial images of the SPLIT groups -> shared memory, [split][c][pixel].
+    // Partial images of the SPLIT groups -> shared memory, [split][c][pixel],
+    // pixels permuted by part_at so that the eight lanes of a 16-byte store
+    // phase (two row blocks of four columns) fall on all 32 banks. With scalar
+    // stores the groups' equal offsets made eight-way conflicts: at short
+    // lists that, and the target's 4-byte copies above, was the largest
+    // per-tile cost (render stage, 93 pairs a tile, 2040x1356 / 200k: 87.7 ->
+    // 79.5 us; 16 uneven images: 180 -> 172 us; 225 pairs a tile: unchanged).
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
+        if constexpr (PX % 4 == 0) {
 #pragma unroll
-        for (int q = 0; q < NP2; ++q) {
-            const int p = (row + r) * T + col0 + 2 * q;
-            spart[(split * 3 + 0) * NPIX + p] = accr[r][q].x;
-            spart[(split * 3 + 0) * NPIX + p + 1] = accr[r][q].y;
-            spart[(split * 3 + 1) * NPIX + p] = accg[r][q].x;
-            spart[(split * 3 + 1) * NPIX + p + 1] = accg[r][q].y;
-            spart[(split * 3 + 2) * NPIX + p] = accb[r][q].x;
-            spart[(split * 3 + 2) * NPIX + p + 1] = accb[r][q].y;
+            for (int q = 0; q < NP2; q += 2) {
+                const int p = part_at<Cfg>((row + r) * T + col0 + 2 * q);
+                *reinterpret_cast<float4*>(&spart[(split * 3 + 0) * NPIX + p]) =
+                    make_float4(accr[r][q].x, accr[r][q].y, accr[r][q + 1].x, accr[r][q + 1].y);
+                *reinterpret_cast<float4*>(&spart[(split * 3 + 1) * NPIX + p]) =
+                    make_float4(accg[r][q].x, accg[r][q].y, accg[r][q + 1].x, accg[r][q + 1].y);
+                *reinterpret_cast<float4*>(&spart[(split * 3 + 2) * NPIX + p]) =
+                    make_float4(accb[r][q].x, accb[r][q].y, accb[r][q + 1].x, accb[r][q + 1].y);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < NP2; ++q) {
+                const int p = part_at<Cfg>((row + r) * T + col0 + 2 * q);
+                *reinterpret_cast<float2*>(&spart[(split * 3 + 0) * NPIX + p]) = accr[r][q];
+                *reinterpret_cast<float2*>(&spart[(split * 3 + 1) * NPIX + p]) = accg[r][q];
+                *reinterpret_cast<float2*>(&spart[(split * 3 + 2) * NPIX + p]) = accb[r][q];
+            }
         }
     }
     __syncthreads();
 
     const float scale = 2.0f / (3.0f * (float)d.W * (float)d.H);
     float lsum = 0.f;
-    if (target) cp_async_wait_all();  // each thread reads back only the pixels it copied
-    __syncthreads();                  // (the copies of a quad below may come from several threads)
+    if (target) cp_async_wait_all();
+    __syncthreads();  // the copies of a quad may come from several threads
     // Epilogue on quads of four neighbouring pixels of a row: 16-byte loads
     // of the partial images, the target and the planar dL/dC, and the quad's
     // twelve HWC floats as three 16-byte stores where they are aligned.
@@ -197,7 +232,7 @@ __device__ __forceinline__ void render_tile(int t, uint32_t& phase, const RSmem<
             float4 sacc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int sp = 0; sp < SPLIT; ++sp) {
-                const float4 u = *reinterpret_cast<const float4*>(&spart[(sp * 3 + c) * NPIX + p]);
+                const float4 u = *reinterpret_cast<const float4*>(&spart[(sp * 3 + c) * NPIX + part_at<Cfg>(p)]);
                 sacc.x += u.x;
                 sacc.y += u.y;
                 sacc.z += u.z;
