@@ -57,12 +57,14 @@ __device__ void zero_job(const ZeroJob& zj) {
 __global__ void __launch_bounds__(kProjBlock) k_project(ParamsIn P, Batch B, float4* __restrict__ rec,
                                                         int4* __restrict__ rect, int32_t* __restrict__ cnt,
                                                         int64_t* __restrict__ blk_sum, ZeroJob zj,
-                                                        uint32_t* __restrict__ M, uint32_t* __restrict__ chunk_sum) {
-    constexpr int CPB = kProjBlock / kCmChunk;  // count-matrix chunks per projection block
-    static_assert(kProjBlock % kCmChunk == 0, "a projection block holds whole count-matrix chunks");
+                                                        uint32_t* __restrict__ M, uint32_t* __restrict__ chunk_sum,
+                                                        int chunk) {
+    constexpr int kMaxCpb = kProjBlock / kCmMinChunk;
+    static_assert(kProjBlock % kCmMinChunk == 0, "a projection block holds whole count-matrix chunks");
+    const int CPB = M ? kProjBlock / chunk : 1;  // count-matrix chunks per projection block
     extern __shared__ uint32_t s_h[];  // with M: [CPB][total_tiles] tile histograms of the block's chunks
     __shared__ int64_t s_warp[32];
-    __shared__ uint32_t s_tot[CPB];
+    __shared__ uint32_t s_tot[kMaxCpb];
     pdl_wait();
     zero_job(zj);
     if (M) {
@@ -213,23 +215,23 @@ __global__ void __launch_bounds__(kProjBlock) k_project(ParamsIn P, Batch B, flo
         rect[g] = r;
         cnt[g] = c;
         if (M && c > 0) {  // count-matrix rows of the fit path (see bin_cm.cu)
-            const int half = threadIdx.x / kCmChunk;
-            uint32_t* h = s_h + half * B.total_tiles;
+            const int row = threadIdx.x / chunk;
+            uint32_t* h = s_h + row * B.total_tiles;
             for (int ty = r.y; ty < r.w; ++ty)
                 for (int tx = r.x; tx < r.z; ++tx) atomicAdd(&h[d.tile_base + ty * d.tw + tx], 1u);
-            atomicAdd(&s_tot[half], (uint32_t)c);
+            atomicAdd(&s_tot[row], (uint32_t)c);
         }
     }
     const int64_t tot = block_sum<int64_t>((int64_t)c, s_warp);  // its barriers also complete the histograms
     if (threadIdx.x == 0 && blk_sum) blk_sum[blockIdx.x] = tot;
     if (M) {
-        const int nchunks = (B.total_gauss + kCmChunk - 1) / kCmChunk;
+        const int nchunks = (B.total_gauss + chunk - 1) / chunk;
         for (int q = 0; q < CPB; ++q) {
-            const int chunk = CPB * blockIdx.x + q;
-            if (chunk >= nchunks) break;
-            uint32_t* row = M + (size_t)chunk * B.total_tiles;
+            const int r = CPB * blockIdx.x + q;
+            if (r >= nchunks) break;
+            uint32_t* row = M + (size_t)r * B.total_tiles;
             for (int i = threadIdx.x; i < B.total_tiles; i += blockDim.x) row[i] = s_h[q * B.total_tiles + i];
-            if (threadIdx.x == 0) chunk_sum[chunk] = s_tot[q];
+            if (threadIdx.x == 0) chunk_sum[r] = s_tot[q];
         }
     }
 }
@@ -651,7 +653,8 @@ BinWs bin_ws_layout(void* base, int64_t n, int64_t capacity, int total_tiles, bo
     const RadixPlan rp = radix_plan(total_tiles);
     const int64_t nblk = std::max<int64_t>(1, (n + kProjBlock - 1) / kProjBlock);
     const int64_t sblk = std::max<int64_t>(1, (capacity + kSortTile - 1) / kSortTile);
-    const int64_t nchunks = std::max<int64_t>(1, (n + kCmChunk - 1) / kCmChunk);
+    const int chunk = cm_chunk(n);
+    const int64_t nchunks = std::max<int64_t>(1, (n + chunk - 1) / chunk);
     const int64_t cap = std::max<int64_t>(1, capacity);
     char* b = static_cast<char*>(base);
     size_t off = 0;
@@ -662,6 +665,7 @@ BinWs bin_ws_layout(void* base, int64_t n, int64_t capacity, int total_tiles, bo
     };
     BinWs w{};
     w.cm_path = cm_applies(n, total_tiles);
+    w.chunk = chunk;
     w.blk_sum = static_cast<int64_t*>(take(nblk * sizeof(int64_t)));
     if (w.cm_path) {
         w.cm = static_cast<uint32_t*>(take((size_t)nchunks * total_tiles * 4));
@@ -686,11 +690,12 @@ BinWs bin_ws_layout(void* base, int64_t n, int64_t capacity, int total_tiles, bo
 }
 
 cudaError_t launch_project(const ParamsIn& P, const Batch& B, float4* rec, int4* rect, int32_t* cnt,
-                           int64_t* blk_sum, const ZeroJob& zj, cudaStream_t s, uint32_t* cm, uint32_t* chunk_sum) {
+                           int64_t* blk_sum, const ZeroJob& zj, cudaStream_t s, const BinWs* ws) {
+    const bool cm = ws && ws->cm_path;
     const int nblk = std::max(1, (B.total_gauss + kProjBlock - 1) / kProjBlock);
-    const size_t smem = cm ? (size_t)(kProjBlock / kCmChunk) * B.total_tiles * 4 : 0;
-    return launch_pdl(k_project, dim3(nblk), dim3(kProjBlock), smem, s, P, B, rec, rect, cnt, blk_sum, zj, cm,
-                      chunk_sum);
+    const size_t smem = cm ? (size_t)(kProjBlock / ws->chunk) * B.total_tiles * 4 : 0;
+    return launch_pdl(k_project, dim3(nblk), dim3(kProjBlock), smem, s, P, B, rec, rect, cnt, blk_sum, zj,
+                      cm ? ws->cm : nullptr, cm ? ws->chunk_sum : nullptr, cm ? ws->chunk : kProjBlock);
 }
 
 cudaError_t launch_bin(const int4* rect, const int32_t* cnt, const float4* rec, const Batch& B, int64_t capacity,

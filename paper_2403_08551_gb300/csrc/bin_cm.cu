@@ -1,7 +1,7 @@
 // bin_cm.cu -- tile binning as a stable counting sort over a count matrix,
 // used when the batch has few tiles (cm_applies).
 //
-// The Gaussians are cut into chunks of kCmChunk consecutive indices. With
+// The Gaussians are cut into chunks of 128 or 256 consecutive indices. With
 // M[b][t] = number of Gaussians of chunk b whose rect covers tile t, the
 // sorted position of the pair (t, g), g in chunk b, is
 //   start[t] + sum_{b' < b} M[b'][t] + #{g' in chunk b : g' < g, t in rect(g')}
@@ -13,7 +13,8 @@
 //             scratch when asked.
 //   k_colscan one block per 16 tiles: column prefix sums over the chunks
 //             (P[b][t] = sum_{b' < b} M[b'][t], written over M) and the
-//             column totals tot[t]; no block waits on another.
+//             column totals tot[t]; no block waits on another. Left out when
+//             M is small (kCmScanCells).
 //   k_place   one block per chunk (two warps per 32 Gaussians): every block
 //             scans the column totals itself (start = exclusive scan of tot
 //             over the at most kCmMaxTiles tiles); a lane mask per 32
@@ -32,6 +33,7 @@ namespace {
 
 constexpr int kCmSlabs = 32;                   // k_colscan: row slabs per tile (one warp scans them)
 constexpr int kCmScanThreads = kCmGroupTiles * kCmSlabs;  // k_colscan: one thread per (tile, slab)
+constexpr int kCmScanCells = 8192;             // counts up to which no k_colscan is launched
 constexpr int kCmRowRegs = 24;                 // k_colscan: rows a lane keeps in registers between passes
 
 __device__ __forceinline__ void zero_words(uint32_t* p, int64_t n) {
@@ -48,12 +50,13 @@ __device__ __forceinline__ bool rect_ok(const int4& r, const ImgDesc& d, int c) 
 
 // Chunk layout shared by k_count and k_place: per Gaussian of the chunk its
 // rect, image tile base and tile-row width, and the exclusive prefix of the
-// pair counts (off[0..kCmChunk], emission order inside the chunk).
+// pair counts (off[0..CH], emission order inside the chunk).
+template <int CH>
 struct ChunkSmem {
-    int off[kCmChunk + 1];
-    int4 rect[kCmChunk];
-    int2 img[kCmChunk];      // (tile_base, tw)
-    float inv_w[kCmChunk];  // 1 / rect width, correctly rounded
+    int off[CH + 1];
+    int4 rect[CH];
+    int2 img[CH];      // (tile_base, tw)
+    float inv_w[CH];  // 1 / rect width, correctly rounded
 };
 
 // Pairs are spread over the lanes of the warp that owns their Gaussians:
@@ -75,7 +78,8 @@ __device__ __forceinline__ int warp_owner(int woff, int p) {
     return lo;
 }
 
-__device__ __forceinline__ int pair_tile(const ChunkSmem& cs, int li, int j) {
+template <int CH>
+__device__ __forceinline__ int pair_tile(const ChunkSmem<CH>& cs, int li, int j) {
     const int4 r = cs.rect[li];
     const int w = r.z - r.x;
     const int q = __float2int_rz(((float)j + 0.5f) * cs.inv_w[li]);
@@ -84,14 +88,15 @@ __device__ __forceinline__ int pair_tile(const ChunkSmem& cs, int li, int j) {
 
 // Loads this thread's Gaussian (count, rect, image) into the chunk layout
 // and returns its count (0 for a bad rect or a negative count, with *bad
-// set). Threads kCmChunk and above of a larger block hold no Gaussian and
+// set). Threads CH and above of a larger block hold no Gaussian and
 // only take part in the scan. The block scan carries a second sum in its
 // upper 32 bits: `hi` in, its inclusive block prefix out in *hi_incl. Ends
 // with the block scan's barrier.
+template <int CH>
 __device__ __forceinline__ int load_chunk(const int4* __restrict__ rect, const int32_t* __restrict__ cnt,
-                                          const Batch& B, int g, ChunkSmem& cs, uint64_t* s_warp, bool* bad,
+                                          const Batch& B, int g, ChunkSmem<CH>& cs, uint64_t* s_warp, bool* bad,
                                           uint32_t hi = 0u, uint32_t* hi_incl = nullptr) {
-    const bool holds = threadIdx.x < kCmChunk;
+    const bool holds = threadIdx.x < CH;
     const bool in = holds && g < B.total_gauss;
     int c = in ? cnt[g] : 0;
     int4 r = in ? rect[g] : make_int4(0, 0, 0, 0);  // issued with the count: no dependent load
@@ -122,16 +127,17 @@ __device__ __forceinline__ int load_chunk(const int4* __restrict__ rect, const i
 }
 
 // ---------------------------------------------------------------------------
-// Count: block = chunk b (kCmChunk threads, one Gaussian each). Every pair
+// Count: block = chunk b (CH threads, one Gaussian each). Every pair
 // adds one to the chunk's shared tile histogram, which is written as row b
 // of M (all tiles, zeros included); chunk_sum[b] = the chunk's pair count.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kCmChunk) k_count(const int4* __restrict__ rect, const int32_t* __restrict__ cnt,
+template <int CH>
+__global__ void __launch_bounds__(CH) k_count(const int4* __restrict__ rect, const int32_t* __restrict__ cnt,
                                                     Batch B, uint32_t* __restrict__ M,
                                                     uint32_t* __restrict__ chunk_sum, uint32_t* __restrict__ zero,
                                                     int64_t zero_n) {
     extern __shared__ uint32_t s_h[];  // [total_tiles]
-    __shared__ ChunkSmem cs;
+    __shared__ ChunkSmem<CH> cs;
     __shared__ uint64_t s_warp[32];
     pdl_wait();
     if (zero) zero_words(zero, zero_n);
@@ -139,8 +145,8 @@ __global__ void __launch_bounds__(kCmChunk) k_count(const int4* __restrict__ rec
     const int b = blockIdx.x;
     for (int i = threadIdx.x; i < Tn; i += blockDim.x) s_h[i] = 0u;
     bool bad;
-    const int c = load_chunk(rect, cnt, B, b * kCmChunk + threadIdx.x, cs, s_warp, &bad);  // k_place raises the error
-    const int total = cs.off[kCmChunk];
+    const int c = load_chunk(rect, cnt, B, b * CH + threadIdx.x, cs, s_warp, &bad);  // k_place raises the error
+    const int total = cs.off[CH];
     {
         const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
         const int woff = cs.off[threadIdx.x] - cs.off[w0];
@@ -261,12 +267,13 @@ __global__ void __launch_bounds__(kCmScanThreads) k_colscan(uint32_t* __restrict
 // over the grid: the tile id over its range) and, in block 0, K, k_max and
 // the capacity check.
 // ---------------------------------------------------------------------------
-constexpr int kPlaceThreads = 2 * kCmChunk;
-constexpr int kTilesPerThread = kCmMaxTiles / kPlaceThreads;
-constexpr int kPlaceSmemWords = kCmChunk / 32 + 2;  // per tile: lane masks, P row, start
-static_assert(kCmMaxTiles % (4 * kPlaceThreads) == 0, "whole uint4 loads of the tile totals per thread");
+template <int CH>
+constexpr int place_smem_words() { return CH / 32 + 2; }  // per tile: lane masks, P row, start
 
-__global__ void __launch_bounds__(kPlaceThreads) k_place(const int4* __restrict__ rect, const int32_t* __restrict__ cnt,
+// SCAN: P still holds the counts M of a few chunks and every block sums its
+// columns itself (no k_colscan).
+template <int CH, bool SCAN>
+__global__ void __launch_bounds__(2 * CH) k_place(const int4* __restrict__ rect, const int32_t* __restrict__ cnt,
                                                          const float4* __restrict__ rec, Batch B,
                                                          const uint32_t* __restrict__ P,
                                                          const uint32_t* __restrict__ tot,
@@ -276,12 +283,15 @@ __global__ void __launch_bounds__(kPlaceThreads) k_place(const int4* __restrict_
                                                          float4* __restrict__ rec_binned, uint32_t* __restrict__ emit,
                                                          int64_t* __restrict__ pair_off, int64_t* __restrict__ k_dev,
                                                          int64_t* __restrict__ k_max, uint32_t* __restrict__ status) {
-    constexpr int NG = kCmChunk / 32;  // lane groups
+    constexpr int kPlaceThreads = 2 * CH;
+    constexpr int kTilesPerThread = kCmMaxTiles / kPlaceThreads;
+    static_assert(kCmMaxTiles % (4 * kPlaceThreads) == 0, "whole uint4 loads of the tile totals per thread");
+    constexpr int NG = CH / 32;  // lane groups
     constexpr int kRowLoads = (kCmMaxTiles + kPlaceThreads - 1) / kPlaceThreads;
     // [NG][total_tiles] lane masks, [total_tiles] P row (+ start), [total_tiles + 1] start
     extern __shared__ uint32_t s_dyn[];
-    __shared__ ChunkSmem cs;
-    __shared__ float4 s_rec[kCmChunk][2];
+    __shared__ ChunkSmem<CH> cs;
+    __shared__ float4 s_rec[CH][2];
     __shared__ uint64_t s_warp[32];
     __shared__ int64_t s_warp64[32];
     pdl_wait();
@@ -290,20 +300,41 @@ __global__ void __launch_bounds__(kPlaceThreads) k_place(const int4* __restrict_
     uint32_t* s_p = s_dyn + NG * Tn;
     uint32_t* s_start = s_p + Tn;
     const int b = blockIdx.x;
-    const bool holds = threadIdx.x < kCmChunk;  // threads holding a Gaussian of the chunk
-    const int g = b * kCmChunk + threadIdx.x;
+    const bool holds = threadIdx.x < CH;  // threads holding a Gaussian of the chunk
+    const int g = b * CH + threadIdx.x;
     // Independent loads first: the chunk's row of P, this thread's tile
     // totals, the chunk totals below b and this Gaussian's record.
-    const uint32_t* prow = P + (size_t)b * Tn;
-#pragma unroll
-    for (int i = 0; i < kRowLoads; ++i) {
-        const int idx = threadIdx.x + i * kPlaceThreads;
-        if (idx < Tn) s_p[idx] = prow[idx];
-    }
     const int t0 = threadIdx.x * kTilesPerThread;
     uint32_t tt[kTilesPerThread];
+    if constexpr (SCAN) {
+        for (int idx = threadIdx.x; idx < Tn; idx += kPlaceThreads) {
+            uint32_t below = 0, all = 0;
+            for (int r0 = 0; r0 < nchunks; r0 += 8) {  // eight predicated loads in flight
+                uint32_t u[8];
 #pragma unroll
-    for (int i = 0; i < kTilesPerThread; i += 4) {
+                for (int q = 0; q < 8; ++q) u[q] = r0 + q < nchunks ? P[(size_t)(r0 + q) * Tn + idx] : 0u;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    all += u[q];
+                    below += r0 + q < b ? u[q] : 0u;
+                }
+            }
+            s_p[idx] = below;
+            s_start[idx] = all;  // the totals, until the starts replace them
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kTilesPerThread; ++i) tt[i] = t0 + i < Tn ? s_start[t0 + i] : 0u;
+    } else {
+        const uint32_t* prow = P + (size_t)b * Tn;
+#pragma unroll
+        for (int i = 0; i < kRowLoads; ++i) {
+            const int idx = threadIdx.x + i * kPlaceThreads;
+            if (idx < Tn) s_p[idx] = prow[idx];
+        }
+    }
+#pragma unroll
+    for (int i = 0; !SCAN && i < kTilesPerThread; i += 4) {
         if (t0 + i + 3 < Tn) {
             const uint4 q = *reinterpret_cast<const uint4*>(tot + t0 + i);
             tt[i] = q.x;
@@ -352,7 +383,7 @@ __global__ void __launch_bounds__(kPlaceThreads) k_place(const int4* __restrict_
     if (holds) {
         const int off = cs.off[threadIdx.x];
         if (g < B.total_gauss) pair_off[g] = pre + off;
-        if (b == nchunks - 1 && threadIdx.x == kCmChunk - 1) pair_off[B.total_gauss] = pre + off + c;
+        if (b == nchunks - 1 && threadIdx.x == CH - 1) pair_off[B.total_gauss] = pre + off + c;
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = warp >> 1, p0 = 32 * (warp & 1), w0 = 32 * grp;
@@ -394,7 +425,7 @@ __global__ void __launch_bounds__(kPlaceThreads) k_place(const int4* __restrict_
         uint32_t pos = s_p[t] + __popc(s_m[grp * Tn + t] & ((1u << l) - 1u));
         for (int v = 0; v < grp; ++v) pos += __popc(s_m[v * Tn + t]);
         if ((int64_t)pos >= capacity) return;  // dropped; block 0 raises the capacity error
-        ids[pos] = (uint32_t)(b * kCmChunk + w0 + l);
+        ids[pos] = (uint32_t)(b * CH + w0 + l);
         if (emit) emit[pos] = (uint32_t)(pre + cs.off[w0 + l] + j);
         if (rec_binned) {
             if (v8) {
@@ -438,33 +469,67 @@ __global__ void __launch_bounds__(kPlaceThreads) k_place(const int4* __restrict_
 }  // namespace
 
 bool cm_applies(int64_t n, int total_tiles) {
-    const int64_t nchunks = std::max<int64_t>(1, (n + kCmChunk - 1) / kCmChunk);
-    return total_tiles >= 1 && total_tiles <= kCmMaxTiles && nchunks * total_tiles <= kCmMaxCells;
+    const int64_t rows = std::max<int64_t>(1, (n + 127) / 128);
+    return total_tiles >= 1 && total_tiles <= kCmMaxTiles && rows * total_tiles <= kCmMaxCells;
 }
+
+// Larger chunks mean fewer rows of M to scan and fewer blocks that each load a
+// row and scan the tile totals: 128 -> 256 takes binning from 19.5 to 17.8 us
+// at 768x512 / 70,000 (render pass 43.8 -> 40.9) and the 640x480 / 40,000 pass
+// from 34.8 to 33.8. Few Gaussians would leave too few blocks: at 256x256 /
+// 2,000 the step takes 34.1 us with 256 and 32.8 with 128; at 10,000 both are
+// equal, at 20,000 the render pass is 1.4 us faster with 256.
+int cm_chunk(int64_t n) { return n <= 8192 ? 128 : 256; }
+
+namespace {
+
+template <int CH>
+cudaError_t bin_cm(const int4* rect, const int32_t* cnt, const float4* rec, const Batch& B, int64_t capacity,
+                   const BinWs& ws, bool prepared, uint32_t* keys, uint32_t* ids, int2* ranges, float4* rec_binned,
+                   uint32_t* emit, int64_t* pair_off, int64_t* k_dev, int64_t* k_max, uint32_t* status,
+                   cudaStream_t s) {
+    const int n = B.total_gauss;
+    const int Tn = B.total_tiles;
+    const int nchunks = std::max(1, (n + CH - 1) / CH);
+    cudaError_t e = cudaSuccess;
+    if (!prepared) {
+        e = launch_pdl(k_count<CH>, dim3(nchunks), dim3(CH), (size_t)Tn * 4, s, rect, cnt, B, ws.cm, ws.chunk_sum,
+                       ws.zero, ws.zero_words);
+        if (e != cudaSuccess) return e;
+    }
+    // Few counts: the placement blocks sum the columns themselves, which saves
+    // a launch (256x256 / 2,000: step 34.9 -> 32.8 us with 16 x 256 counts;
+    // 40 x 256 counts: no difference, 40 x 576: 2 us slower).
+    const bool scan = (int64_t)nchunks * Tn <= kCmScanCells;
+    if (!scan) {
+        const int groups = (Tn + kCmGroupTiles - 1) / kCmGroupTiles;
+        e = launch_pdl(k_colscan, dim3(groups), dim3(kCmScanThreads), 0, s, ws.cm, nchunks, Tn, ws.tile_tot);
+        if (e != cudaSuccess) return e;
+    }
+    // lane masks, P row and starts: above the default 48 KB window
+    const auto kern = scan ? k_place<CH, true> : k_place<CH, false>;
+    e = smem_optin(reinterpret_cast<const void*>(kern), place_smem_words<CH>() * kCmMaxTiles * 4 + 4);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kern, dim3(nchunks), dim3(2 * CH), (size_t)(place_smem_words<CH>() * Tn + 1) * 4, s, rect, cnt,
+                      rec, B, ws.cm, ws.tile_tot, ws.chunk_sum, nchunks, capacity, keys, ids, ranges, rec_binned, emit,
+                      pair_off, k_dev, k_max, status);
+}
+
+}  // namespace
 
 cudaError_t launch_bin_cm(const int4* rect, const int32_t* cnt, const float4* rec, const Batch& B, int64_t capacity,
                           const BinWs& ws, bool prepared, uint32_t* keys, uint32_t* ids, int2* ranges,
                           float4* rec_binned, uint32_t* emit, int64_t* pair_off, int64_t* k_dev, int64_t* k_max,
                           uint32_t* status, cudaStream_t s) {
-    const int n = B.total_gauss;
-    const int Tn = B.total_tiles;
-    const int nchunks = std::max(1, (n + kCmChunk - 1) / kCmChunk);
-    const int groups = (Tn + kCmGroupTiles - 1) / kCmGroupTiles;
-    cudaError_t e = cudaSuccess;
-    if (!prepared) {
-        e = launch_pdl(k_count, dim3(nchunks), dim3(kCmChunk), (size_t)Tn * 4, s, rect, cnt, B, ws.cm, ws.chunk_sum,
-                       ws.zero, ws.zero_words);
-        if (e != cudaSuccess) return e;
+    auto go = [&](auto fn) {
+        return fn(rect, cnt, rec, B, capacity, ws, prepared, keys, ids, ranges, rec_binned, emit, pair_off, k_dev,
+                  k_max, status, s);
+    };
+    switch (ws.chunk) {
+        case 128: return go(bin_cm<128>);
+        case 256: return go(bin_cm<256>);
+        default: return cudaErrorInvalidValue;
     }
-    e = launch_pdl(k_colscan, dim3(groups), dim3(kCmScanThreads), 0, s, ws.cm, nchunks, Tn, ws.tile_tot);
-    if (e != cudaSuccess) return e;
-    // lane masks, P row and starts: up to 48 KB dynamic + the static layout,
-    // above the default 48 KB window
-    e = smem_optin(reinterpret_cast<const void*>(k_place), kPlaceSmemWords * kCmMaxTiles * 4 + 4);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(k_place, dim3(nchunks), dim3(kPlaceThreads), (size_t)(kPlaceSmemWords * Tn + 1) * 4, s, rect,
-                      cnt, rec, B, ws.cm, ws.tile_tot, ws.chunk_sum, nchunks, capacity, keys, ids, ranges, rec_binned,
-                      emit, pair_off, k_dev, k_max, status);
 }
 
 }  // namespace gi

@@ -78,8 +78,7 @@ cudaError_t enqueue_forward(gi_fit* f, cudaStream_t s, bool train) {
     cudaError_t e = train ? mark(f, 0, s) : cudaSuccess;
     if (e == cudaSuccess) {
         NvtxRange r("gi:formation");
-        e = launch_project(params_aos(f->params), f->B, f->rec, f->rect, f->cnt, f->bws.blk_sum, zj, s, f->bws.cm,
-                           f->bws.chunk_sum);
+        e = launch_project(params_aos(f->params), f->B, f->rec, f->rect, f->cnt, f->bws.blk_sum, zj, s, &f->bws);
     }
     if (e == cudaSuccess && train) e = mark(f, 1, s);
     if (e == cudaSuccess) {

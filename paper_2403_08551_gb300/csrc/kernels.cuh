@@ -41,9 +41,11 @@ constexpr int kHistReplicas = 8;       // copies of each pass's digit histogram 
 constexpr int kSortTile = kSortThreads * kSortItems;  // keys per onesweep block
 constexpr int kSortStageBytes = kSortTile * 8;          // keys + values staged in digit order
 
-// Count-matrix binning (bin_cm.cu): chunks of kCmChunk Gaussians; used when
-// the batch has at most kCmMaxTiles tiles and chunks x tiles <= kCmMaxCells.
-constexpr int kCmChunk = 128;
+// Count-matrix binning (bin_cm.cu): chunks of cm_chunk(n) Gaussians; used when
+// the batch has at most kCmMaxTiles tiles and 128-Gaussian rows x tiles <=
+// kCmMaxCells.
+int cm_chunk(int64_t n);
+constexpr int kCmMinChunk = 128;
 constexpr int kCmGroupTiles = 16;  // count-matrix column scan: tiles per block
 constexpr int kCmMaxTiles = 2048;
 constexpr int64_t kCmMaxCells = int64_t(1) << 20;
@@ -55,6 +57,7 @@ bool cm_applies(int64_t n, int total_tiles);
 // [chunks][tiles], chunk_sum [chunks], tile_tot [tiles] (column totals).
 struct BinWs {
     bool cm_path;
+    int chunk;            // Gaussians per count-matrix row
     int64_t* blk_sum;     // [ceil(n / kProjBlock)]
     uint32_t* keys_tmp;   // [capacity]          (radix)
     uint32_t* vals_tmp;   // [capacity]          (radix)
@@ -74,11 +77,10 @@ struct BinWs {
 BinWs bin_ws_layout(void* base, int64_t n, int64_t capacity, int total_tiles, bool with_owner = true);
 
 // Launchers (stream-ordered, no host synchronisation).
-// With cm != null (count-matrix binning to follow) the projection also
-// writes the count-matrix rows and chunk totals of its Gaussians.
+// With ws on the count-matrix path (that binning to follow) the projection
+// also writes the count-matrix rows and chunk totals of its Gaussians.
 cudaError_t launch_project(const ParamsIn& P, const Batch& B, float4* rec, int4* rect, int32_t* cnt,
-                           int64_t* blk_sum, const ZeroJob& zj, cudaStream_t s, uint32_t* cm = nullptr,
-                           uint32_t* chunk_sum = nullptr);
+                           int64_t* blk_sum, const ZeroJob& zj, cudaStream_t s, const BinWs* ws = nullptr);
 // emit (nullable): [capacity] emission index of each sorted pair.
 cudaError_t launch_bin(const int4* rect, const int32_t* cnt, const float4* rec, const Batch& B,
                        int64_t capacity, const BinWs& ws, bool blk_sum_ready, uint32_t* keys,
