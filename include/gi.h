@@ -86,7 +86,8 @@ typedef struct {
 /* ABI version: 8 (gi_fit_desc gained param_mode, optimizer, beta3, lr_halve_every in 2,
  * cov_mode in 3, the codec fine-tuning fields in 4, opacity_mode and opacity_logits in 5;
  * gi_fit_set_target_source in 6; gi_codec_decode in 7; gi_fit_count_pairs and the
- * GI_FIT_KEYS .. GI_FIT_MEANS16 pointers in 8). */
+ * GI_FIT_KEYS .. GI_FIT_MEANS16 pointers in 8; gi_render_pass and gi_rasterize_* were
+ * added to 8 without changing it). */
 GI_API int32_t gi_abi_version(void);
 GI_API const char* gi_last_error(void);
 GI_API const char* gi_status_string(int32_t status);
@@ -177,6 +178,39 @@ GI_API gi_status gi_bin_tiles_noalloc(const int32_t* rect, const int32_t* cnt, c
  * ---------------------------------------------------------------------- */
 GI_API gi_status gi_render(const float* rec_binned, const int32_t* ranges, gi_image img, const float* target,
                     float* out, float* dl_dout, double* loss_sum, gi_stream stream);
+
+/* ------------------------------------------------------------------------
+ * gi_render_pass -- gi_project, gi_bin_tiles and gi_render (no target) in one
+ * call with the same outputs bit for bit and fewer launches: the projection
+ * also writes the counts that the binning starts from. Arguments as there;
+ * ws of gi_bin_workspace_size() bytes, all outputs required.
+ * ---------------------------------------------------------------------- */
+GI_API gi_status gi_render_pass(const float* means, const float* chol, const float* color, int32_t n, gi_image img,
+                                int64_t capacity, void* ws, size_t ws_bytes, float* rec, int32_t* rect, int32_t* cnt,
+                                uint32_t* keys, uint32_t* ids, int32_t* ranges, float* rec_binned, int64_t* pair_off,
+                                int64_t* k_dev, float* out, gi_stream stream);
+
+/* ------------------------------------------------------------------------
+ * gi_rasterize_forward / gi_rasterize_backward -- the differentiable render
+ * of an autograd program: gi_render_pass, then gi_render_backward of the same
+ * pass, with everything the backward needs kept in one caller-owned buffer.
+ *   state, state_bytes  *forward_bytes of gi_rasterize_size() (device,
+ *                       256-byte aligned); keep it unchanged until the backward.
+ *   pairs (host)        K. If K > capacity the image is incomplete and
+ *                       GI_DEVERR_CAPACITY is raised, as with gi_bin_tiles.
+ *   ws, ws_bytes        scratch of *backward_bytes.
+ * The forward waits for its binning to learn K (not for the render behind
+ * it) and so cannot be captured; the backward waits for nothing.
+ * ---------------------------------------------------------------------- */
+GI_API gi_status gi_rasterize_size(int32_t n, gi_image img, int64_t capacity, size_t* forward_bytes,
+                                   size_t* backward_bytes);
+GI_API gi_status gi_rasterize_forward(const float* means, const float* chol, const float* color, int32_t n,
+                                      gi_image img, int64_t capacity, void* state, size_t state_bytes, float* out,
+                                      int64_t* pairs, gi_stream stream);
+GI_API gi_status gi_rasterize_backward(const void* state, size_t state_bytes, const float* chol, int32_t n,
+                                       gi_image img, int64_t capacity, const float* dl_dout, void* ws,
+                                       size_t ws_bytes, float* g_means, float* g_chol, float* g_color,
+                                       gi_stream stream);
 
 /* ------------------------------------------------------------------------
  * gi_render_backward -- gradients of the render (App. A.1) chained through

@@ -199,23 +199,57 @@ def codec_decode(stream: dict):
 
 class GIRender(torch.autograd.Function):
     """Differentiable render: forward runs formation, binning and Eq. 7;
-    backward recomputes the weights per tile (no per-pixel state saved)."""
+    backward recomputes the weights per tile (no per-pixel state saved).
+    Each is one library call on buffers carved from one allocation (one host
+    synchronisation in the forward, for the pair count, while the render
+    already runs). A pair count above the first guess repeats the pass once
+    with the exact capacity."""
 
     @staticmethod
     def forward(ctx, means, chol, color, W: int, H: int, tile: int = 16):
-        rec, rect, cnt = project(means, chol, color, W, H, tile)
-        bins = bin_tiles(rect, cnt, rec, W, H, tile)
-        out, _, _ = render(bins, W, H, tile)
-        ctx.save_for_backward(chol.detach().contiguous(), rect, cnt)
-        ctx.bins = bins
-        ctx.meta = (W, H, tile)
+        lib = L.load()
+        means = _dev(means, torch.float32, "means")
+        chol = _dev(chol, torch.float32, "chol")
+        color = _dev(color, torch.float32, "color")
+        n = means.shape[0]
+        img = _img(W, H, tile)
+        stream = L.stream_handle()
+        fwd, bwd, pairs = ctypes.c_size_t(0), ctypes.c_size_t(0), ctypes.c_int64(0)
+        cap = max(4096, 8 * n)
+        out = None
+        for _ in range(2):
+            L.check(lib.gi_rasterize_size(n, img, cap, ctypes.byref(fwd), ctypes.byref(bwd)), "gi_rasterize_size")
+            state = torch.empty((fwd.value,), dtype=torch.uint8, device=means.device)
+            if out is None:
+                out = torch.empty((H, W, 3), dtype=torch.float32, device=means.device)
+            L.check(lib.gi_rasterize_forward(L.ptr(means) if n else None, L.ptr(chol) if n else None,
+                                             L.ptr(color) if n else None, n, img, cap, L.ptr(state), fwd.value,
+                                             L.ptr(out), ctypes.byref(pairs), stream), "gi_rasterize_forward")
+            if pairs.value <= cap:
+                break
+            device_errors(clear=True)  # drop the capacity bit raised by the short guess
+            cap = pairs.value
+        else:
+            raise L.GIError("gi_rasterize_forward: capacity retry failed")
+        ctx.save_for_backward(chol.detach())
+        ctx.state = state
+        ctx.meta = (n, img, cap, fwd.value, bwd.value)
         return out
 
     @staticmethod
     def backward(ctx, grad_out):
-        chol, rect, cnt = ctx.saved_tensors
-        W, H, tile = ctx.meta
-        gm, gl, gc, _ = render_backward(ctx.bins, rect, cnt, chol, grad_out.contiguous(), W, H, tile)
+        chol, = ctx.saved_tensors
+        n, img, cap, fwd, bwd = ctx.meta
+        dl = _dev(grad_out, torch.float32, "dl_dout")
+        chol = _dev(chol, torch.float32, "chol")
+        dev = chol.device
+        ws = torch.empty((bwd,), dtype=torch.uint8, device=dev)
+        gm = torch.empty((n, 2), dtype=torch.float32, device=dev)
+        gl = torch.empty((n, 3), dtype=torch.float32, device=dev)
+        gc = torch.empty((n, 3), dtype=torch.float32, device=dev)
+        L.check(L.load().gi_rasterize_backward(L.ptr(ctx.state), fwd, L.ptr(chol), n, img, cap, L.ptr(dl), L.ptr(ws),
+                                               bwd, L.ptr(gm), L.ptr(gl), L.ptr(gc), L.stream_handle()),
+                "gi_rasterize_backward")
         return gm, gl, gc, None, None, None
 
 
@@ -591,16 +625,12 @@ class Renderer:
         self.out = torch.empty((H, W, 3), dtype=f32, device=device)
 
     def __call__(self, means, chol, color):
-        lib = L.load()
-        img = _img(self.W, self.H, self.tile)
-        s = L.stream_handle()
-        L.check(lib.gi_project(L.ptr(means), L.ptr(chol), L.ptr(color), self.n, img, L.ptr(self.rec),
-                               L.ptr(self.rect), L.ptr(self.cnt), s), "gi_project")
-        L.check(lib.gi_bin_tiles(L.ptr(self.rect), L.ptr(self.cnt), L.ptr(self.rec), self.n, img, self.capacity,
-                                 L.ptr(self.ws), self.ws_bytes, L.ptr(self.keys), L.ptr(self.ids), L.ptr(self.ranges),
-                                 L.ptr(self.rec_binned), L.ptr(self.pair_off), L.ptr(self.k_dev), s), "gi_bin_tiles")
-        L.check(lib.gi_render(L.ptr(self.rec_binned), L.ptr(self.ranges), img, None, L.ptr(self.out), None, None, s),
-                "gi_render")
+        L.check(L.load().gi_render_pass(L.ptr(means), L.ptr(chol), L.ptr(color), self.n,
+                                        _img(self.W, self.H, self.tile), self.capacity, L.ptr(self.ws), self.ws_bytes,
+                                        L.ptr(self.rec), L.ptr(self.rect), L.ptr(self.cnt), L.ptr(self.keys),
+                                        L.ptr(self.ids), L.ptr(self.ranges), L.ptr(self.rec_binned),
+                                        L.ptr(self.pair_off), L.ptr(self.k_dev), L.ptr(self.out), L.stream_handle()),
+                "gi_render_pass")
         return self.out
 
 

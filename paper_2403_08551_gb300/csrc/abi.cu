@@ -41,6 +41,107 @@ Batch single(const gi_image& img, int32_t n) {
     return b;
 }
 
+// Buffers of a fused formation + binning + render.
+struct RasterBufs {
+    float4* rec;
+    int4* rect;
+    int32_t* cnt;
+    uint32_t *keys, *ids;
+    int2* ranges;
+    float4* rec_binned;
+    uint32_t* emit;  // nullable
+    int64_t *pair_off, *k_dev;
+    BinWs ws;
+};
+
+size_t up256(size_t x) { return (x + 255) / 256 * 256; }
+size_t raster_partial_bytes(int64_t capacity) { return up256((size_t)capacity * 32); }
+size_t raster_dl_bytes(const gi_image& img) {
+    return up256((size_t)single(img, 0).total_tiles * img.tile * img.tile * 12);
+}
+
+// Carve-up of gi_rasterize_forward's state; bytes = its size.
+RasterBufs raster_layout(void* base, int32_t n, const gi_image& img, int64_t capacity, size_t& bytes) {
+    RasterBufs b{};
+    const int tiles = single(img, n).total_tiles;
+    b.ws = bin_ws_layout(base, n, capacity, tiles);
+    const size_t N = (size_t)(n > 0 ? n : 1), cap = (size_t)capacity;
+    char* p = static_cast<char*>(base);
+    size_t off = up256(b.ws.bytes);
+    auto take = [&](size_t x) -> void* {
+        const size_t o = off;
+        off += up256(x);
+        return p ? p + o : nullptr;
+    };
+    b.rec = static_cast<float4*>(take(N * 32));
+    b.rect = static_cast<int4*>(take(N * 16));
+    b.cnt = static_cast<int32_t*>(take(N * 4));
+    b.keys = static_cast<uint32_t*>(take(cap * 4));
+    b.ids = static_cast<uint32_t*>(take(cap * 4));
+    b.ranges = static_cast<int2*>(take((size_t)tiles * 8));
+    b.rec_binned = static_cast<float4*>(take(cap * 32));
+    b.emit = static_cast<uint32_t*>(take(cap * 4));
+    b.pair_off = static_cast<int64_t*>(take((N + 1) * 8));
+    b.k_dev = static_cast<int64_t*>(take(8));
+    bytes = off;
+    return b;
+}
+
+// Formation (which also writes the counts the binning starts from) and binning.
+cudaError_t enqueue_form_bin(const float* means, const float* chol, const float* color, const Batch& B,
+                             int64_t capacity, const RasterBufs& b, cudaStream_t s) {
+    ZeroJob zj{};
+    zj.p[0] = b.ws.zero;
+    zj.n32[0] = b.ws.zero_words;
+    zj.p[1] = reinterpret_cast<uint32_t*>(b.ranges);
+    zj.n32[1] = (int64_t)B.total_tiles * 2;
+    const cudaError_t e = launch_project(params_soa(means, chol, color), B, b.rec, b.rect, b.cnt, b.ws.blk_sum, zj, s,
+                                         &b.ws);
+    if (e != cudaSuccess) return e;
+    return launch_bin(b.rect, b.cnt, b.rec, B, capacity, b.ws, true, b.keys, b.ids, b.ranges, b.rec_binned, b.emit,
+                      b.pair_off, b.k_dev, nullptr, device_status(), s);
+}
+
+cudaError_t enqueue_plain_render(const Batch& B, const RasterBufs& b, float* out, cudaStream_t s) {
+    return launch_render(b.rec_binned, b.ranges, B, nullptr, out, nullptr, nullptr, nullptr, nullptr, device_status(),
+                         s);
+}
+
+// The pinned word and event a host thread waits for a pair count with: one of
+// each per thread, for the device it last used, given back when it ends.
+struct PairsWait {
+    int dev = -1;
+    int64_t* k = nullptr;
+    cudaEvent_t ev = nullptr;
+    void drop() {
+        if (ev) cudaEventDestroy(ev);
+        if (k) cudaFreeHost(k);
+        ev = nullptr;
+        k = nullptr;
+        dev = -1;
+    }
+    ~PairsWait() { drop(); }  // after the runtime has shut down both calls only return an error
+};
+
+PairsWait* pairs_wait() {
+    thread_local PairsWait w;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    if (w.dev != dev) {
+        w.drop();
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, sizeof(int64_t), cudaHostAllocDefault) != cudaSuccess) return nullptr;
+        w.k = static_cast<int64_t*>(p);
+        if (cudaEventCreateWithFlags(&w.ev, cudaEventDisableTiming) != cudaSuccess) {
+            w.ev = nullptr;
+            w.drop();
+            return nullptr;
+        }
+        w.dev = dev;
+    }
+    return &w;
+}
+
 #define GI_REQUIRE(cond, ...)                                   \
     do {                                                        \
         if (!(cond)) return set_error(GI_ERR_INVALID_ARG, __VA_ARGS__); \
@@ -268,6 +369,116 @@ gi_status gi_render_backward(const float* rec_binned, const uint32_t* keys, cons
         e = launch_reduce(partial, pair_off, cnt, capacity, n, params_soa(nullptr, chol, nullptr), g_means, g_chol,
                           g_color, g_conic, nullptr, nullptr, nullptr, nullptr, nullptr, B, s);
     if (e != cudaSuccess) return set_cuda_error(e, "gi_render_backward");
+    return GI_OK;
+}
+
+gi_status gi_render_pass(const float* means, const float* chol, const float* color, int32_t n, gi_image img,
+                         int64_t capacity, void* ws, size_t ws_bytes, float* rec, int32_t* rect, int32_t* cnt,
+                         uint32_t* keys, uint32_t* ids, int32_t* ranges, float* rec_binned, int64_t* pair_off,
+                         int64_t* k_dev, float* out, gi_stream stream) {
+    NvtxRange nvtx_("gi_render_pass");
+    if (n <= 0) {  // nothing to form: the separate calls (and their checks of n)
+        gi_status st = gi_project(means, chol, color, n, img, rec, rect, cnt, stream);
+        if (st == GI_OK)
+            st = gi_bin_tiles(rect, cnt, rec, n, img, capacity, ws, ws_bytes, keys, ids, ranges, rec_binned, pair_off,
+                              k_dev, stream);
+        return st == GI_OK ? gi_render(rec_binned, ranges, img, nullptr, out, nullptr, nullptr, stream) : st;
+    }
+    gi_status st = check_image(img, "gi_render_pass");
+    if (st != GI_OK) return st;
+    GI_REQUIRE(capacity >= 1 && capacity <= kMaxCapacity, "gi_render_pass: capacity %lld outside [1, 2^30)",
+               (long long)capacity);
+    GI_REQUIRE(means && chol && color && ws && rec && rect && cnt && keys && ids && ranges && rec_binned && pair_off &&
+                   k_dev && out,
+               "gi_render_pass: NULL pointer");
+    GI_REQUIRE(aligned(ws, 256) && aligned(rec, 16) && aligned(rect, 16) && aligned(ranges, 16) &&
+                   aligned(rec_binned, 16) && aligned(pair_off, 8) && aligned(k_dev, 8) && aligned(means, 4) &&
+                   aligned(chol, 4) && aligned(color, 4) && aligned(cnt, 4) && aligned(keys, 4) && aligned(ids, 4) &&
+                   aligned(out, 4),
+               "gi_render_pass: misaligned pointer");
+    const BinWs w = bin_ws_layout(ws, n, capacity, single(img, n).total_tiles);
+    GI_REQUIRE(ws_bytes >= w.bytes, "gi_render_pass: workspace %zu bytes < %zu needed", ws_bytes, w.bytes);
+    const RasterBufs b{reinterpret_cast<float4*>(rec), reinterpret_cast<int4*>(rect), cnt, keys, ids,
+                       reinterpret_cast<int2*>(ranges), reinterpret_cast<float4*>(rec_binned), nullptr, pair_off, k_dev,
+                       w};
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    cudaError_t e = enqueue_form_bin(means, chol, color, single(img, n), capacity, b, s);
+    if (e == cudaSuccess) e = enqueue_plain_render(single(img, 0), b, out, s);
+    if (e != cudaSuccess) return set_cuda_error(e, "gi_render_pass");
+    return GI_OK;
+}
+
+gi_status gi_rasterize_size(int32_t n, gi_image img, int64_t capacity, size_t* forward_bytes, size_t* backward_bytes) {
+    gi_status st = check_image(img, "gi_rasterize_size");
+    if (st != GI_OK) return st;
+    GI_REQUIRE(forward_bytes && backward_bytes, "gi_rasterize_size: NULL pointer");
+    GI_REQUIRE(n >= 0 && capacity >= 1 && capacity <= kMaxCapacity,
+               "gi_rasterize_size: bad n (%d) or capacity (%lld)", n, (long long)capacity);
+    size_t bytes = 0;
+    raster_layout(nullptr, n, img, capacity, bytes);
+    *forward_bytes = bytes;
+    *backward_bytes = raster_partial_bytes(capacity) + raster_dl_bytes(img);
+    return GI_OK;
+}
+
+gi_status gi_rasterize_forward(const float* means, const float* chol, const float* color, int32_t n, gi_image img,
+                               int64_t capacity, void* state, size_t state_bytes, float* out, int64_t* pairs,
+                               gi_stream stream) {
+    NvtxRange nvtx_("gi_rasterize_forward");
+    size_t need = 0, unused = 0;
+    gi_status st = gi_rasterize_size(n, img, capacity, &need, &unused);
+    if (st != GI_OK) return st;
+    GI_REQUIRE(state && out && pairs && (n == 0 || (means && chol && color)), "gi_rasterize_forward: NULL pointer");
+    GI_REQUIRE(aligned(state, 256) && aligned(means, 4) && aligned(chol, 4) && aligned(color, 4) && aligned(out, 4),
+               "gi_rasterize_forward: misaligned pointer");
+    GI_REQUIRE(state_bytes >= need, "gi_rasterize_forward: state %zu bytes < %zu needed", state_bytes, need);
+    const RasterBufs b = raster_layout(state, n, img, capacity, need);
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    *pairs = 0;
+    if (n == 0) {
+        st = gi_bin_tiles(nullptr, nullptr, nullptr, 0, img, capacity, state, b.ws.bytes, b.keys, b.ids,
+                          reinterpret_cast<int32_t*>(b.ranges), reinterpret_cast<float*>(b.rec_binned), b.pair_off,
+                          b.k_dev, stream);
+        return st == GI_OK ? gi_render(reinterpret_cast<float*>(b.rec_binned), reinterpret_cast<int32_t*>(b.ranges),
+                                       img, nullptr, out, nullptr, nullptr, stream)
+                           : st;
+    }
+    PairsWait* w = pairs_wait();
+    if (!w) return set_error(GI_ERR_NO_MEMORY, "gi_rasterize_forward: no pinned word or event");
+    cudaError_t e = enqueue_form_bin(means, chol, color, single(img, n), capacity, b, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(w->k, b.k_dev, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaEventRecord(w->ev, s);
+    if (e == cudaSuccess) e = enqueue_plain_render(single(img, 0), b, out, s);
+    if (e == cudaSuccess) e = cudaEventSynchronize(w->ev);
+    if (e != cudaSuccess) return set_cuda_error(e, "gi_rasterize_forward");
+    *pairs = *w->k;
+    return GI_OK;
+}
+
+gi_status gi_rasterize_backward(const void* state, size_t state_bytes, const float* chol, int32_t n, gi_image img,
+                                int64_t capacity, const float* dl_dout, void* ws, size_t ws_bytes, float* g_means,
+                                float* g_chol, float* g_color, gi_stream stream) {
+    NvtxRange nvtx_("gi_rasterize_backward");
+    size_t fwd = 0, bwd = 0;
+    gi_status st = gi_rasterize_size(n, img, capacity, &fwd, &bwd);
+    if (st != GI_OK) return st;
+    if (n == 0) return GI_OK;
+    GI_REQUIRE(state && chol && dl_dout && ws && g_means && g_chol && g_color, "gi_rasterize_backward: NULL pointer");
+    GI_REQUIRE(aligned(state, 256) && aligned(ws, 256), "gi_rasterize_backward: misaligned pointer");
+    GI_REQUIRE(state_bytes >= fwd && ws_bytes >= bwd, "gi_rasterize_backward: state %zu or workspace %zu bytes < %zu, %zu",
+               state_bytes, ws_bytes, fwd, bwd);
+    const RasterBufs b = raster_layout(const_cast<void*>(state), n, img, capacity, fwd);
+    const Batch B = single(img, n);
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    float4* partial = static_cast<float4*>(ws);
+    float* dl_tiled = reinterpret_cast<float*>(static_cast<char*>(ws) + raster_partial_bytes(capacity));
+    cudaError_t e = launch_pack_dl(dl_dout, B, dl_tiled, s);
+    if (e == cudaSuccess)
+        e = launch_backward(b.rec_binned, b.keys, b.emit, dl_tiled, B, b.k_dev, capacity, partial, device_status(), s);
+    if (e == cudaSuccess)
+        e = launch_reduce(partial, b.pair_off, b.cnt, capacity, n, params_soa(nullptr, chol, nullptr), g_means, g_chol,
+                          g_color, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, B, s);
+    if (e != cudaSuccess) return set_cuda_error(e, "gi_rasterize_backward");
     return GI_OK;
 }
 
