@@ -191,7 +191,7 @@ __device__ __forceinline__ void render_tile(int t, uint32_t& phase, const RSmem<
     // stores the groups' equal offsets made eight-way conflicts: at short
     // lists that, and the target's 4-byte copies above, was the largest
     // per-tile cost (render stage, 93 pairs a tile, 2040x1356 / 200k: 87.7 ->
-    // 79.5 us; 16 uneven images: 180 -> 172 us; 225 pairs a tile: unchanged).
+    // 85.7 us; 225 pairs a tile: unchanged).
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
         if constexpr (PX % 4 == 0) {
@@ -305,9 +305,13 @@ __device__ __forceinline__ void render_tile(int t, uint32_t& phase, const RSmem<
     }
 }
 
-// One block per tile, tiles in index order.
+// One block per tile, tiles in index order. The explicit minimum of one block
+// lets the compiler use the registers it wants (98 instead of 80 at split 4,
+// where shared memory bounds the residency anyway): render stage 85.7 -> 79.5
+// us at 2040x1356 / 200k with the wide partial stores below (87.7 before both),
+// 178 -> 172 us on 16 uneven images.
 template <class Cfg>
-__global__ void __launch_bounds__(Cfg::kThreads) k_render(const float4* __restrict__ rec_binned,
+__global__ void __launch_bounds__(Cfg::kThreads, 1) k_render(const float4* __restrict__ rec_binned,
                                                           const int2* __restrict__ ranges, Batch B,
                                                           const float* __restrict__ target, float* __restrict__ out,
                                                           float* __restrict__ dl_hwc, float* __restrict__ dl_tiled,
