@@ -392,9 +392,9 @@ __global__ void __launch_bounds__(kProjBlock) k_emit(const int4* __restrict__ re
 // multi-split (items ordered by (warp, round, lane) = input order, so the
 // ranking is stable), resolves its per-digit global offset with a decoupled
 // look-back over lower tickets (bounded spin), and scatters. A thread owns
-// digits threadIdx.x and threadIdx.x + kSortThreads in the per-digit phases.
+// digit threadIdx.x in the per-digit phases.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortThreads) k_onesweep(
+__global__ void __launch_bounds__(kSortThreads, 1) k_onesweep(
     const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
     uint32_t* __restrict__ vals_out, const int64_t* __restrict__ k_dev, int64_t capacity, int shift, int dbits,
     const uint32_t* __restrict__ hist, uint32_t* __restrict__ lookback, uint32_t* __restrict__ ticket,

@@ -32,7 +32,11 @@ struct RadixPlan {
 RadixPlan radix_plan(int total_tiles);
 
 constexpr int kProjBlock = 256;        // Gaussians per projection / emit block
-constexpr int kSortThreads = 256;      // threads per onesweep block
+// 8,192 keys a block: half the blocks and so half the look-back rounds of 256
+// threads, and at 1 M pairs every SM has at most one (step 308.2 -> 305.8 us at
+// 2040x1356 / 200,000, 731.5 -> 724.2 us on 16 uneven images; 512 x 8: 307.5,
+// 726.9; 1024 x 8: 307.8, 729.3; 512 x 12: 314.4, 728.4).
+constexpr int kSortThreads = 512;      // threads per onesweep block
 constexpr int kSortItems = 16;         // keys per thread
 constexpr int kMaxDigitBits = 9;       // radix digits of at most 9 bits (512 buckets)
 constexpr int kMaxRadix = 1 << kMaxDigitBits;
