@@ -221,10 +221,13 @@ template <int T>
 __global__ void __launch_bounds__(kBwdThreads, 2) k_backward(
     const float4* __restrict__ rec_binned, const uint32_t* __restrict__ keys, const uint32_t* __restrict__ emit,
     const float* __restrict__ dl_tiled, Batch B, const int64_t* __restrict__ k_dev, int64_t capacity,
-    float4* __restrict__ partial, uint32_t* __restrict__ status) {
+    float4* __restrict__ partial, int32_t* __restrict__ step, uint32_t* __restrict__ status) {
     constexpr int TF = tile_floats<T>();
     extern __shared__ float4 s_dyn[];
     pdl_wait();
+    // The optimiser's step counter, read by the kernels behind this one
+    // (counted here, the reduction's blocks need no last-block election).
+    if (step && blockIdx.x == 0 && threadIdx.x == 0) ++*step;
     const int K = (int)min(*k_dev, capacity);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     BwdWarpSmem<T>& w = reinterpret_cast<BwdWarpSmem<T>*>(s_dyn)[wib];
@@ -464,10 +467,10 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(const float4* __restr
     // 1/sqrt(1 - b3^t); [3] = learning-rate factor of the halving schedule.
     __shared__ float s_bc[4];
     pdl_wait();
-    // The step counter's load is issued here and used after the partials are
-    // summed, so no load below waits for it.
-    int step_prev = 0;
-    if (ADAM && threadIdx.x == 0) step_prev = *cfg.step;
+    // The step counter's load (the backward has advanced it) is issued here
+    // and used after the partials are summed, so no load below waits for it.
+    int step = 0;
+    if (ADAM && threadIdx.x == 0) step = *cfg.step;
     const int gblocks = (int)max(1, (n + kReduceThreads - 1) / kReduceThreads);
     // With loss_tile the first B.nimg blocks sum the images' squared errors
     // (first, so that they start in the first wave) and the Gaussian blocks
@@ -477,8 +480,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(const float4* __restr
     if (gb < 0) {
         // image b = blockIdx.x: its tiles' partials in tile order, eight loads
         // in flight per thread, combined in a fixed order, then a fixed
-        // reduction tree (reproducible run to run); then the block counts
-        // itself done like the others
+        // reduction tree (reproducible run to run)
         __shared__ double s_lw[32];
         {
             const int b = (int)blockIdx.x;
@@ -495,15 +497,6 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(const float4* __restr
             double tot = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
             tot = block_sum<double>(tot, s_lw);
             if (threadIdx.x == 0) loss[b] = tot;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            if (atomicAdd(cfg.done, 1u) == gridDim.x - 1) {
-                *cfg.step = step_prev + 1;
-                *cfg.done = 0u;
-                __threadfence();
-            }
         }
         return;
     }
@@ -579,7 +572,6 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(const float4* __restr
     }
     if (ADAM) {
         if (threadIdx.x == 0) {
-            const int step = step_prev + 1;
             s_step = step;
             s_bc[0] = 1.f / (1.f - powf(cfg.beta1, (float)step));
             if (cfg.optimizer == 1) {
@@ -779,20 +771,6 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(const float4* __restr
         }
     }
     if (ADAM && CODEC) codec_block_partials(B.codec, cv_gb, cv_j, cv_r, cv_commit, gb, gblocks);
-    if (ADAM) {
-        // The last block to finish advances the step counter (every block has
-        // read it by then).
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            const unsigned prev = atomicAdd(cfg.done, 1u);
-            if (prev == gridDim.x - 1) {
-                *cfg.step = s_step;
-                *cfg.done = 0u;
-                __threadfence();
-            }
-        }
-    }
 }
 
 // Codec sums, stage 2: block v adds row v of the per-block partials in a
@@ -920,7 +898,7 @@ int backward_blocks_per_sm() {
 template <int T>
 cudaError_t launch_backward_t(const float4* rec_binned, const uint32_t* keys, const uint32_t* emit,
                               const float* dl_tiled, const Batch& B, const int64_t* k_dev, int64_t capacity,
-                              float4* partial, uint32_t* status, cudaStream_t s) {
+                              float4* partial, uint32_t* status, cudaStream_t s, int32_t* step) {
     cudaError_t e = smem_optin(reinterpret_cast<const void*>(k_backward<T>), (int)backward_smem<T>());
     if (e != cudaSuccess) return e;
     // persistent: one wave of resident blocks (no more than the tasks need)
@@ -928,19 +906,19 @@ cudaError_t launch_backward_t(const float4* rec_binned, const uint32_t* keys, co
     const int64_t full = (int64_t)sm_count() * backward_blocks_per_sm<T>();
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(full, (tasks + kBwdWarps - 1) / kBwdWarps));
     return launch_pdl(k_backward<T>, dim3(blocks), dim3(kBwdThreads), backward_smem<T>(), s, rec_binned, keys, emit,
-                      dl_tiled, B, k_dev, capacity, partial, status);
+                      dl_tiled, B, k_dev, capacity, partial, step, status);
 }
 
 }  // namespace
 
 cudaError_t launch_backward(const float4* rec_binned, const uint32_t* keys, const uint32_t* emit,
                             const float* dl_tiled, const Batch& B, const int64_t* k_dev, int64_t capacity,
-                            float4* partial, uint32_t* status, cudaStream_t s) {
+                            float4* partial, uint32_t* status, cudaStream_t s, int32_t* step) {
     if (capacity <= 0) return cudaSuccess;
     switch (B.tile) {
-        case 8: return launch_backward_t<8>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s);
-        case 16: return launch_backward_t<16>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s);
-        case 32: return launch_backward_t<32>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s);
+        case 8: return launch_backward_t<8>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s, step);
+        case 16: return launch_backward_t<16>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s, step);
+        case 32: return launch_backward_t<32>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s, step);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -38,7 +38,7 @@ struct gi_fit {
     int4* rect = nullptr;
     int32_t* cnt = nullptr;
     int64_t *pair_off = nullptr, *k_dev = nullptr, *k_max = nullptr;
-    uint32_t *keys = nullptr, *ids = nullptr, *emit = nullptr, *done = nullptr;
+    uint32_t *keys = nullptr, *ids = nullptr, *emit = nullptr;
     int2* ranges = nullptr;
     double* loss = nullptr;
     double* loss_tile = nullptr;  // [tiles] squared error per tile of the last step
@@ -107,9 +107,9 @@ cudaError_t enqueue_step(gi_fit* f, cudaStream_t s) {
         NvtxRange r("gi:backward");
         e = f->B.opac.mode == 2
                 ? launch_backward_blend(f->rec_binned, f->ids, f->ranges, f->rect, f->pair_off, f->B, f->out,
-                                        f->dl_tiled, f->capacity, f->partial, device_status(), s)
+                                        f->dl_tiled, f->capacity, f->partial, device_status(), s, f->step)
                 : launch_backward(f->rec_binned, f->keys, f->emit, f->dl_tiled, f->B, f->k_dev, f->capacity,
-                                  f->partial, device_status(), s);
+                                  f->partial, device_status(), s, f->step);
     }
     if (e == cudaSuccess) e = mark(f, 4, s);
     if (e == cudaSuccess) {
@@ -279,7 +279,7 @@ gi_status gi_fit_create(const gi_fit_desc* d, gi_stream stream, gi_fit** out) {
         up256((size_t)f->capacity * 4), up256((size_t)f->capacity * 4),  // 15-16 keys ids
         up256((size_t)tiles * 8),                               // 17 ranges
         up256((size_t)d->n_images * 8),                         // 18 loss
-        256,                                                    // 19 step, done
+        256,                                                    // 19 step
         up256(probe.bytes),                                     // 20 bin ws
         d->optimizer == 1 ? up256((size_t)N * 32) : 0,          // 21 Adan n
         d->optimizer == 1 ? up256((size_t)N * 32) : 0,          // 22 Adan g_prev
@@ -340,7 +340,6 @@ gi_status gi_fit_create(const gi_fit_desc* d, gi_stream stream, gi_fit** out) {
     }
     f->loss = reinterpret_cast<double*>(at(18));
     f->step = reinterpret_cast<int32_t*>(at(19));
-    f->done = reinterpret_cast<uint32_t*>(at(19) + 16);
     f->bws = bin_ws_layout(at(20), N, f->capacity, (int)tiles);
     f->B.many = d->n_images > 1 ? f->d_desc : nullptr;
 
@@ -351,7 +350,6 @@ gi_status gi_fit_create(const gi_fit_desc* d, gi_stream stream, gi_fit** out) {
     f->adam.beta2 = d->beta2;
     f->adam.eps = d->eps;
     f->adam.step = f->step;
-    f->adam.done = f->done;
     f->adam.optimizer = d->optimizer;
     f->adam.beta3 = d->beta3;
     f->adam.lr_halve_every = d->lr_halve_every;

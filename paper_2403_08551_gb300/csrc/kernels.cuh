@@ -122,13 +122,15 @@ cudaError_t launch_render_blend(const float4* rec_binned, const uint32_t* ids, c
                                 cudaStream_t s);
 cudaError_t launch_backward_blend(const float4* rec_binned, const uint32_t* ids, const int2* ranges, const int4* rect,
                                   const int64_t* pair_off, const Batch& B, const float* out, const float* dl_tiled,
-                                  int64_t capacity, float4* partial, uint32_t* status, cudaStream_t s);
+                                  int64_t capacity, float4* partial, uint32_t* status, cudaStream_t s,
+                                  int32_t* step = nullptr);
 
 // Backward: per-pair partial sums (8 floats per pair at its emission index
-// emit[k], written by the binning or by launch_emit_index).
+// emit[k], written by the binning or by launch_emit_index). Both backwards
+// advance *step (nullable), the optimiser's step counter.
 cudaError_t launch_backward(const float4* rec_binned, const uint32_t* keys, const uint32_t* emit,
                             const float* dl_tiled, const Batch& B, const int64_t* k_dev, int64_t capacity,
-                            float4* partial, uint32_t* status, cudaStream_t s);
+                            float4* partial, uint32_t* status, cudaStream_t s, int32_t* step = nullptr);
 cudaError_t launch_emit_index(const uint32_t* keys, const uint32_t* ids, const int4* rect, const int64_t* pair_off,
                               const Batch& B, const int64_t* k_dev, int64_t capacity, uint32_t* emit,
                               uint32_t* status, cudaStream_t s);
@@ -137,8 +139,7 @@ cudaError_t launch_pack_dl(const float* dl_hwc, const Batch& B, float* dl_tiled,
 struct AdamCfg {
     float lr[3];  // means, chol, color
     float beta1, beta2, eps;
-    int32_t* step;  // device counter (1-based step of the update being made = *step + 1)
-    uint32_t* done; // device counter for the last-block step increment
+    int32_t* step;  // device counter: the step of the update being made (the backward has advanced it)
     int32_t optimizer;       // 0: Adam; 1: Adan (beta1, beta2, beta3 decay m, v, n)
     float beta3;             // Adan
     int32_t lr_halve_every;  // every learning rate halves every this many steps; 0 = never
