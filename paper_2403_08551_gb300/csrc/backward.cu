@@ -396,25 +396,53 @@ __device__ void codec_block_partials(const CodecCfg& Q, const float (&gb)[6], co
         const float w = warp_sum(commit);
         if (lane == 0) s_cv[nv - 1] = w;
     }
+    // Up to 8 entries a stage (the paper's size): each lane spreads its residual
+    // over 32 slots (4 x entry + count or component) and one reduce-scatter of
+    // 31 shuffles leaves slot l's warp sum in lane l, in the order of the
+    // butterfly below; larger codebooks take one butterfly per entry in use.
+    // (768x512 / 70,000, 2 x 8 entries: 480 -> 62 shuffles a warp.)
+    const bool small = Q.size <= 8;
 #pragma unroll
     for (int m = 0; m < kCodecMaxStages; ++m) {
-        if (m < Q.stages) {
-            for (int j = 0; j < Q.size; ++j) {
+        if (m >= Q.stages) continue;
+        if (small) {
+            float v[32];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
                 const bool mine = jj[m] == j;
-                const unsigned mask = __ballot_sync(0xffffffffu, mine);
-                float c0 = 0.f, c1 = 0.f, c2 = 0.f;
-                if (mask) {  // warp-uniform
-                    c0 = warp_sum(mine ? rr[m][0] : 0.f);
-                    c1 = warp_sum(mine ? rr[m][1] : 0.f);
-                    c2 = warp_sum(mine ? rr[m][2] : 0.f);
+                v[4 * j] = mine ? 1.f : 0.f;
+                v[4 * j + 1] = mine ? rr[m][0] : 0.f;
+                v[4 * j + 2] = mine ? rr[m][1] : 0.f;
+                v[4 * j + 3] = mine ? rr[m][2] : 0.f;
+            }
+#pragma unroll
+            for (int w = 16; w >= 1; w >>= 1) {  // keep w slots
+                const bool up = (lane & w) != 0;
+#pragma unroll
+                for (int i = 0; i < w; ++i) {
+                    const float send = up ? v[i] : v[i + w];
+                    const float keep = up ? v[i + w] : v[i];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
                 }
-                if (lane == 0) {
-                    float* o = &s_cv[6 + (m * Q.size + j) * 4];
-                    o[0] = (float)__popc(mask);
-                    o[1] = c0;
-                    o[2] = c1;
-                    o[3] = c2;
-                }
+            }
+            if ((lane >> 2) < Q.size) s_cv[6 + m * Q.size * 4 + lane] = v[0];
+            continue;
+        }
+        for (int j = 0; j < Q.size; ++j) {
+            const bool mine = jj[m] == j;
+            const unsigned mask = __ballot_sync(0xffffffffu, mine);
+            float c0 = 0.f, c1 = 0.f, c2 = 0.f;
+            if (mask) {  // warp-uniform
+                c0 = warp_sum(mine ? rr[m][0] : 0.f);
+                c1 = warp_sum(mine ? rr[m][1] : 0.f);
+                c2 = warp_sum(mine ? rr[m][2] : 0.f);
+            }
+            if (lane == 0) {
+                float* o = &s_cv[6 + (m * Q.size + j) * 4];
+                o[0] = (float)__popc(mask);
+                o[1] = c0;
+                o[2] = c1;
+                o[3] = c2;
             }
         }
     }
@@ -786,8 +814,29 @@ __global__ void __launch_bounds__(kCodecSumThreads) k_codec_update(CodecCfg Q, A
     unsigned* ticket = Q.ticket;
     __shared__ double s_w[32];
     __shared__ bool s_last;
+    constexpr int kMB = kCodecMaxEntries;
+    __shared__ double s_cnt[kMB];
+    __shared__ double s_sum[kMB * 3];
     pdl_wait();
     const int v = blockIdx.x;
+    const int MB = Q.stages * Q.size;
+    const int step = *cfg.step;  // the backward has advanced it
+    float corr1 = 0.f, corr2 = 0.f, corr3 = 0.f;  // bias corrections
+    // What the last block needs besides the totals is fetched by every block of
+    // a small codebook before its own sum (the last one is not known yet), so
+    // that it does not wait for it afterwards.
+    const bool early = MB <= 64;
+    auto fetch = [&]() {
+        for (int i = threadIdx.x; i < MB; i += blockDim.x) s_cnt[i] = Q.ema_count[i];
+        for (int i = threadIdx.x; i < 3 * MB; i += blockDim.x) s_sum[i] = Q.ema_total[i];
+        if (threadIdx.x < 6) {
+            corr1 = 1.f / (1.f - powf(cfg.beta1, (float)step));
+            corr2 = cfg.optimizer == 1 ? 1.f / (1.f - powf(cfg.beta2, (float)step))
+                                       : rsqrtf(1.f - powf(cfg.beta2, (float)step));
+            corr3 = cfg.optimizer == 1 ? rsqrtf(1.f - powf(cfg.beta3, (float)step)) : 0.f;
+        }
+    };
+    if (early) fetch();
     double acc = 0.0;
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x) acc += Q.part[(size_t)v * nblocks + b];
     acc = block_sum<double>(acc, s_w);
@@ -803,15 +852,10 @@ __global__ void __launch_bounds__(kCodecSumThreads) k_codec_update(CodecCfg Q, A
     const int t = threadIdx.x;
     // Everything the update reads is loaded in parallel first (a chain of
     // dependent global read-modify-writes would cost a round trip each).
-    constexpr int kMB = kCodecMaxEntries;
     __shared__ double s_tot[kCodecMaxVals];
-    __shared__ double s_cnt[kMB];
-    __shared__ double s_sum[kMB * 3];
     __shared__ double s_stage[kCodecMaxStages];
-    const int MB = Q.stages * Q.size;
     for (int i = t; i < nv; i += blockDim.x) s_tot[i] = __ldcg(tot + i);
-    for (int i = t; i < MB; i += blockDim.x) s_cnt[i] = Q.ema_count[i];
-    for (int i = t; i < 3 * MB; i += blockDim.x) s_sum[i] = Q.ema_total[i];
+    if (!early) fetch();
     __syncthreads();
     {
         const double d = (double)Q.decay;
@@ -842,7 +886,6 @@ __global__ void __launch_bounds__(kCodecSumThreads) k_codec_update(CodecCfg Q, A
     if (t < 6) {
         const float gr = (float)s_tot[t];
         Q.out[1 + t] = s_tot[t];
-        const int step = *cfg.step;  // already advanced by the reduction
         const float lr = cfg.lr[1] * (cfg.lr_halve_every > 0 ? ldexpf(1.f, -((step - 1) / cfg.lr_halve_every)) : 1.f);
         float* p = Q.gb;
         float& m = p[6 + t];
@@ -855,15 +898,12 @@ __global__ void __launch_bounds__(kCodecSumThreads) k_codec_update(CodecCfg Q, A
             vv = cfg.beta2 * vv + (1.f - cfg.beta2) * dg;
             const float ge = gr + cfg.beta2 * dg;
             nn = cfg.beta3 * nn + (1.f - cfg.beta3) * ge * ge;
-            const float b1 = 1.f / (1.f - powf(cfg.beta1, (float)step)), b2 = 1.f / (1.f - powf(cfg.beta2, (float)step));
-            const float b3 = rsqrtf(1.f - powf(cfg.beta3, (float)step));
-            p[t] -= lr * (m * b1 + cfg.beta2 * (vv * b2)) / (sqrtf(nn) * b3 + cfg.eps);
+            p[t] -= lr * (m * corr1 + cfg.beta2 * (vv * corr2)) / (sqrtf(nn) * corr3 + cfg.eps);
             gp = gr;
         } else {
             m = cfg.beta1 * m + (1.f - cfg.beta1) * gr;
             vv = cfg.beta2 * vv + (1.f - cfg.beta2) * gr * gr;
-            const float b1 = 1.f / (1.f - powf(cfg.beta1, (float)step)), b2 = rsqrtf(1.f - powf(cfg.beta2, (float)step));
-            p[t] -= (lr * b1) * m / (sqrtf(vv) * b2 + cfg.eps);
+            p[t] -= (lr * corr1) * m / (sqrtf(vv) * corr2 + cfg.eps);
         }
     } else if (t == 64) {
         Q.out[0] = n > 0 ? s_tot[nv - 1] / ((double)n * Q.size) : 0.0;

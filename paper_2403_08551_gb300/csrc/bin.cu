@@ -216,7 +216,11 @@ __global__ void __launch_bounds__(kProjBlock) k_project(ParamsIn P, Batch B, flo
             auto code8 = [](float q) { return (unsigned char)(q >= 0.f && q <= 255.f ? (int)q : 0); };
             Q.codes[g] = make_uchar4(code8(q0), code8(q1), code8(q2), 0);
             float r0 = cr, r1 = cg, r2 = cb;
+            // The colour is the exact sum of the chosen entries rounded once: one
+            // FP32 addition does that for two stages, FP64 sums for more.
             double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+            float f0 = 0.f, f1 = 0.f, f2 = 0.f;
+            const bool two = Q.stages <= 2;
             for (int m = 0; m < Q.stages; ++m) {
                 const float* cbk = Q.codebooks + (size_t)m * Q.size * 3;
                 const int j = rvq_pick(cbk, Q.size, r0, r1, r2);
@@ -225,13 +229,19 @@ __global__ void __launch_bounds__(kProjBlock) k_project(ParamsIn P, Batch B, flo
                 r0 = __fsub_rn(r0, e0);
                 r1 = __fsub_rn(r1, e1);
                 r2 = __fsub_rn(r2, e2);
-                s0 = __dadd_rn(s0, (double)e0);
-                s1 = __dadd_rn(s1, (double)e1);
-                s2 = __dadd_rn(s2, (double)e2);
+                if (two) {
+                    f0 = __fadd_rn(f0, e0);
+                    f1 = __fadd_rn(f1, e1);
+                    f2 = __fadd_rn(f2, e2);
+                } else {
+                    s0 = __dadd_rn(s0, (double)e0);
+                    s1 = __dadd_rn(s1, (double)e1);
+                    s2 = __dadd_rn(s2, (double)e2);
+                }
             }
-            cr = (float)s0;
-            cg = (float)s1;
-            cb = (float)s2;
+            cr = two ? f0 : (float)s0;
+            cg = two ? f1 : (float)s1;
+            cb = two ? f2 : (float)s2;
         }
         int4 r = make_int4(0, 0, 0, 0);
         float4 r0 = make_float4(mx, my, 0.f, 0.f), r1 = make_float4(0.f, cr, cg, cb);
