@@ -138,8 +138,18 @@ __global__ void __launch_bounds__(kProjBlock) k_project(ParamsIn P, Batch B, flo
     extern __shared__ uint32_t s_h[];  // with M: [CPB][total_tiles] tile histograms of the block's chunks
     __shared__ int64_t s_warp[32];
     __shared__ uint32_t s_tot[kMaxCpb];
+    // codec: the codebooks' entries, padded (from global memory every thread
+    // waited for each entry's loads in turn: k_project 12.3 -> 9.8 us, step
+    // 114.5 -> 112.1 us at 70,000 Gaussians, 2 x 8 entries)
+    __shared__ float4 s_cb[kCodecMaxEntries];
     pdl_wait();
     zero_job(zj);
+    if (B.codec.bits > 0) {
+        const float* cb = B.codec.codebooks;
+        for (int i = threadIdx.x; i < B.codec.stages * B.codec.size; i += blockDim.x)
+            s_cb[i] = make_float4(cb[3 * i], cb[3 * i + 1], cb[3 * i + 2], 0.f);
+        __syncthreads();
+    }
     if (M) {
         for (int i = threadIdx.x; i < CPB * B.total_tiles; i += blockDim.x) s_h[i] = 0u;
         if (threadIdx.x < CPB) s_tot[threadIdx.x] = 0u;
@@ -222,10 +232,10 @@ __global__ void __launch_bounds__(kProjBlock) k_project(ParamsIn P, Batch B, flo
             float f0 = 0.f, f1 = 0.f, f2 = 0.f;
             const bool two = Q.stages <= 2;
             for (int m = 0; m < Q.stages; ++m) {
-                const float* cbk = Q.codebooks + (size_t)m * Q.size * 3;
+                const float4* cbk = s_cb + m * Q.size;
                 const int j = rvq_pick(cbk, Q.size, r0, r1, r2);
                 Q.idx[(size_t)m * B.total_gauss + g] = (uint8_t)j;
-                const float e0 = cbk[3 * j], e1 = cbk[3 * j + 1], e2 = cbk[3 * j + 2];
+                const float e0 = cbk[j].x, e1 = cbk[j].y, e2 = cbk[j].z;
                 r0 = __fsub_rn(r0, e0);
                 r1 = __fsub_rn(r1, e1);
                 r2 = __fsub_rn(r2, e2);

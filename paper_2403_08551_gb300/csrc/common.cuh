@@ -129,16 +129,18 @@ __device__ __forceinline__ float lsq_quant(float l, float gamma, float beta, flo
 // One greedy RVQ stage (Sec. 3.3, Eq. 10): the entry of cb [size][3] nearest to
 // r, distances ((e0^2 + e1^2) + e2^2) in FP32 with one rounding per operation,
 // scanning upward and moving only on a strictly smaller distance.
-__device__ __forceinline__ float rvq_dist(const float* __restrict__ e, float r0, float r1, float r2) {
-    const float e0 = __fsub_rn(e[0], r0), e1 = __fsub_rn(e[1], r1), e2 = __fsub_rn(e[2], r2);
+__device__ __forceinline__ float rvq_dist(float4 e, float r0, float r1, float r2) {
+    const float e0 = __fsub_rn(e.x, r0), e1 = __fsub_rn(e.y, r1), e2 = __fsub_rn(e.z, r2);
     return __fadd_rn(__fadd_rn(__fmul_rn(e0, e0), __fmul_rn(e1, e1)), __fmul_rn(e2, e2));
 }
 
-__device__ __forceinline__ int rvq_pick(const float* __restrict__ cb, int size, float r0, float r1, float r2) {
+// cb: entries padded to four floats (shared memory, one 16-byte broadcast each).
+__device__ __forceinline__ int rvq_pick(const float4* cb, int size, float r0, float r1, float r2) {
     int best = 0;
-    float bd = rvq_dist(cb, r0, r1, r2);
+    float bd = rvq_dist(cb[0], r0, r1, r2);
+#pragma unroll 4
     for (int j = 1; j < size; ++j) {
-        const float d = rvq_dist(cb + 3 * j, r0, r1, r2);
+        const float d = rvq_dist(cb[j], r0, r1, r2);
         if (d < bd) {
             bd = d;
             best = j;
