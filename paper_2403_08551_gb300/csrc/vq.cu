@@ -75,160 +75,135 @@ __global__ void __launch_bounds__(256) k_vq_decode(const uint16_t* __restrict__ 
     }
 }
 
-// One quad of the fast path below (at most two stages): the four
-// Gaussians' attributes from their index words w[attribute][stage] and the
-// padded codebook rows, then the 16-byte stores.
-__device__ __forceinline__ void vq_store_quad(int q, uint4 h, const uint32_t (&w)[2][2], const float4* srow,
-                                              int stages, int cbs, float4* __restrict__ means,
-                                              float4* __restrict__ chol, float4* __restrict__ color,
-                                              uint32_t* status) {
-    float o[2][4][3];
+constexpr int kVqQuads = 2;  // quads per thread and round of the fast path
+// From this count on, two-stage decodes keep eight copies of the codebook rows
+// in shared memory (lane l reads copy l mod 8, so the eight rows of a 16-byte
+// load phase fall on different banks; 128 KB for 2 x 256 entries, one block of
+// 1024 threads per SM). Random rows otherwise collide about 2.7-fold, which
+// alone takes 18 us of shared-memory time at 3.2 M. Graph-replayed, 2 x 256
+// entries, eight copies / one: 600,000 Gaussians 7.4 / 7.0 us, 800,000 12.5 /
+// 10.6, 1.2 M 14.0 / 15.7, 3.2 M 28.5 / 33.7 (before the staged stores 34.6). One
+// stage gains nothing (25 us either way).
+constexpr int kVqReplicated = 1200000;
+
+// The decoded attribute a (0: Cholesky vector, 1: colour) of a quad from its
+// index words w[stage] and the padded codebook rows: up to two stages as FP32
+// sums (exact), more in FP64, rounded once.
+template <int MAXS>
+__device__ __forceinline__ void vq_quad(const uint32_t (&w)[MAXS], const float4* rows, int copies, int stages,
+                                        int cbs, float (&o)[4][3], uint32_t* status) {
 #pragma unroll
-    for (int a = 0; a < 2; ++a) {
+    for (int j = 0; j < 4; ++j) {
+        float f[3] = {0.f, 0.f, 0.f};
+        double d[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) o[a][j][0] = o[a][j][1] = o[a][j][2] = 0.f;
-#pragma unroll
-        for (int st = 0; st < 2; ++st) {
+        for (int st = 0; st < MAXS; ++st) {
             if (st < stages) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    int i = (w[a][st] >> (8 * j)) & 0xff;
-                    if (i >= cbs) {  // index outside the codebook: skip the read
-                        flag_error(status, kErrBounds);
-                        i = 0;
-                    }
-                    const float4 r = srow[((size_t)a * stages + st) * cbs + i];
-                    o[a][j][0] = __fadd_rn(o[a][j][0], r.x);
-                    o[a][j][1] = __fadd_rn(o[a][j][1], r.y);
-                    o[a][j][2] = __fadd_rn(o[a][j][2], r.z);
+                int i = (w[st] >> (8 * j)) & 0xff;
+                if (i >= cbs) {  // index outside the codebook: skip the read
+                    flag_error(status, kErrBounds);
+                    i = 0;
+                }
+                const float4 r = rows[(st * cbs + i) * copies];
+                if (MAXS <= 2) {
+                    f[0] = __fadd_rn(f[0], r.x);
+                    f[1] = __fadd_rn(f[1], r.y);
+                    f[2] = __fadd_rn(f[2], r.z);
+                } else {
+                    d[0] += (double)r.x;
+                    d[1] += (double)r.y;
+                    d[2] += (double)r.z;
                 }
             }
         }
-    }
-    const uint32_t hw[4] = {h.x, h.y, h.z, h.w};
-    float mf[8];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        mf[2 * j] = __half2float(__ushort_as_half((unsigned short)(hw[j] & 0xffffu)));
-        mf[2 * j + 1] = __half2float(__ushort_as_half((unsigned short)(hw[j] >> 16)));
-    }
-    means[2 * (size_t)q] = make_float4(mf[0], mf[1], mf[2], mf[3]);
-    means[2 * (size_t)q + 1] = make_float4(mf[4], mf[5], mf[6], mf[7]);
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-        float4* dst = (a == 0 ? chol : color) + 3 * (size_t)q;
-        dst[0] = make_float4(o[a][0][0], o[a][0][1], o[a][0][2], o[a][1][0]);
-        dst[1] = make_float4(o[a][1][1], o[a][1][2], o[a][2][0], o[a][2][1]);
-        dst[2] = make_float4(o[a][2][2], o[a][3][0], o[a][3][1], o[a][3][2]);
+        for (int c = 0; c < 3; ++c) o[j][c] = MAXS <= 2 ? f[c] : (float)d[c];
     }
 }
 
-constexpr int kVqQuads = 2;  // quads per thread and round of the fast path (4 measured slower)
-
-// Four consecutive Gaussians per thread when every array is 16-byte aligned
-// (the usual case): the FP16 positions of the four as one 16-byte load, each
-// index plane as one 4-byte load, codebook rows from shared memory as one
-// 16-byte load each (rows padded to four floats), and the outputs as whole
-// 16-byte stores (2 for the positions, 3 for each attribute). Same
-// arithmetic as k_vq_decode.
-__global__ void __launch_bounds__(256) k_vq_decode4(const uint2* __restrict__ means16, const uint8_t* __restrict__ idx,
-                                                    const float* __restrict__ cb, int n, int stages, int cbs,
-                                                    float4* __restrict__ means, float4* __restrict__ chol,
-                                                    float4* __restrict__ color, uint32_t* status) {
-    extern __shared__ float4 srow[];  // [2][stages][cbs] rows (x, y, z, 0)
-    const int nrow = 2 * stages * cbs;
-    for (int i = threadIdx.x; i < nrow; i += blockDim.x)
-        srow[i] = make_float4(cb[3 * i], cb[3 * i + 1], cb[3 * i + 2], 0.f);
-    __syncthreads();
-    const int nq = n >> 2;  // whole quads; the tail is left to k_vq_decode
-    const int stride = gridDim.x * blockDim.x;
-    if (stages <= 2) {
-        // kVqQuads quads per round, every load of the round issued before any
-        // quad is decoded (the loads' latency overlaps)
-        const uint4* M = reinterpret_cast<const uint4*>(means16);
-        for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += kVqQuads * stride) {
-            uint4 h[kVqQuads];
-            uint32_t w[kVqQuads][2][2];
-#pragma unroll
-            for (int u = 0; u < kVqQuads; ++u) {
-                const int qu = q + u * stride;
-                const bool in = qu < nq;
-                h[u] = in ? M[qu] : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                for (int a = 0; a < 2; ++a)
-#pragma unroll
-                    for (int st = 0; st < 2; ++st) {
-                        const uint32_t* I = reinterpret_cast<const uint32_t*>(idx + ((size_t)a * stages + st) * n);
-                        w[u][a][st] = st < stages && in ? I[qu] : 0u;
-                    }
-            }
-#pragma unroll
-            for (int u = 0; u < kVqQuads; ++u)
-                if (q + u * stride < nq)
-                    vq_store_quad(q + u * stride, h[u], w[u], srow, stages, cbs, means, chol, color, status);
-        }
-        return;
+// Four consecutive Gaussians (a quad) per lane when every array is 16-byte
+// aligned (the usual case): the FP16 positions of the four as one 16-byte
+// load, each index plane as one 4-byte load, codebook rows from shared memory
+// as one 16-byte load each (rows padded to four floats). Same arithmetic as
+// k_vq_decode. 80 % of the bytes are written: the positions leave as one
+// 32-byte store per lane, and the 48 bytes of each attribute go through the
+// warp's corner of shared memory so that every store instruction writes 512
+// contiguous bytes (three 16-byte stores 48 bytes apart fill half a sector
+// each; one stage, 3.2 M: 32.5 -> 24.5 us).
+template <int MAXS, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_vq_decode4(const uint4* __restrict__ means16,
+                                                           const uint8_t* __restrict__ idx,
+                                                           const float* __restrict__ cb, int n, int stages, int cbs,
+                                                           float4* __restrict__ means, float4* __restrict__ chol,
+                                                           float4* __restrict__ color, int copies, bool v8,
+                                                           uint32_t* status) {
+    extern __shared__ float4 srow[];  // [2][stages][cbs][copies] rows (x, y, z, 0), then [warps][96]
+    const int nrow = 2 * stages * cbs * copies;
+    for (int i = threadIdx.x; i < nrow; i += blockDim.x) {
+        const int r = i / copies;
+        srow[i] = make_float4(cb[3 * r], cb[3 * r + 1], cb[3 * r + 2], 0.f);
     }
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += stride) {
-        const uint4 h = reinterpret_cast<const uint4*>(means16)[q];  // 4 Gaussians x (x, y) binary16
-        float o[2][4][3];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const float4* rows = srow + (lane & (copies - 1));  // this lane's copy
+    float4* stage = srow + nrow + 96 * (threadIdx.x >> 5);
+    const int nq = n >> 2;
+    const int stride = gridDim.x * blockDim.x;
+    for (int q0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); q0 < nq; q0 += kVqQuads * stride) {
+        // every load of the round is issued before any quad is decoded
+        uint4 h[kVqQuads];
+        uint32_t w[kVqQuads][2][MAXS];
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            if (stages <= 2) {
+        for (int u = 0; u < kVqQuads; ++u) {
+            const int q = q0 + u * stride + lane;
+            const bool in = q < nq;
+            h[u] = in ? means16[q] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) o[a][j][0] = o[a][j][1] = o[a][j][2] = 0.f;
-                for (int s = 0; s < stages; ++s) {
-                    const uint32_t w = reinterpret_cast<const uint32_t*>(idx + ((size_t)a * stages + s) * n)[q];
+            for (int a = 0; a < 2; ++a)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        int i = (w >> (8 * j)) & 0xff;
-                        if (i >= cbs) {  // index outside the codebook: skip the read
-                            flag_error(status, kErrBounds);
-                            i = 0;
-                        }
-                        const float4 r = srow[((size_t)a * stages + s) * cbs + i];
-                        o[a][j][0] = __fadd_rn(o[a][j][0], r.x);
-                        o[a][j][1] = __fadd_rn(o[a][j][1], r.y);
-                        o[a][j][2] = __fadd_rn(o[a][j][2], r.z);
-                    }
+                for (int st = 0; st < MAXS; ++st) {
+                    const uint32_t* I = reinterpret_cast<const uint32_t*>(idx + ((size_t)a * stages + st) * n);
+                    w[u][a][st] = st < stages && in ? I[q] : 0u;
                 }
-            } else {
-                double acc[4][3] = {};
-                for (int s = 0; s < stages; ++s) {
-                    const uint32_t w = reinterpret_cast<const uint32_t*>(idx + ((size_t)a * stages + s) * n)[q];
+        }
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        int i = (w >> (8 * j)) & 0xff;
-                        if (i >= cbs) {
-                            flag_error(status, kErrBounds);
-                            i = 0;
-                        }
-                        const float4 r = srow[((size_t)a * stages + s) * cbs + i];
-                        acc[j][0] += (double)r.x;
-                        acc[j][1] += (double)r.y;
-                        acc[j][2] += (double)r.z;
-                    }
+        for (int u = 0; u < kVqQuads; ++u) {
+            const int qb = q0 + u * stride;  // the warp's first quad
+            if (qb >= nq) break;
+            const int valid = min(32, nq - qb);
+            if (lane < valid) {
+                const uint32_t hw[4] = {h[u].x, h[u].y, h[u].z, h[u].w};
+                float mf[8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    mf[2 * j] = __half2float(__ushort_as_half((unsigned short)(hw[j] & 0xffffu)));
+                    mf[2 * j + 1] = __half2float(__ushort_as_half((unsigned short)(hw[j] >> 16)));
                 }
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    for (int c = 0; c < 3; ++c) o[a][j][c] = (float)acc[j][c];
+                const float4 m0 = make_float4(mf[0], mf[1], mf[2], mf[3]), m1 = make_float4(mf[4], mf[5], mf[6], mf[7]);
+                float4* m = means + 2 * (size_t)(qb + lane);
+                if (v8) {
+                    st_global_v8(m, m0, m1);
+                } else {
+                    m[0] = m0;
+                    m[1] = m1;
+                }
             }
-        }
-        const uint32_t hw[4] = {h.x, h.y, h.z, h.w};
-        float mf[8];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            mf[2 * j] = __half2float(__ushort_as_half((unsigned short)(hw[j] & 0xffffu)));
-            mf[2 * j + 1] = __half2float(__ushort_as_half((unsigned short)(hw[j] >> 16)));
-        }
-        means[2 * (size_t)q] = make_float4(mf[0], mf[1], mf[2], mf[3]);
-        means[2 * (size_t)q + 1] = make_float4(mf[4], mf[5], mf[6], mf[7]);
+            for (int a = 0; a < 2; ++a) {
+                float o[4][3];
+                if (lane < valid) {
+                    vq_quad<MAXS>(w[u][a], rows + a * stages * cbs * copies, copies, stages, cbs, o, status);
+                    stage[3 * lane] = make_float4(o[0][0], o[0][1], o[0][2], o[1][0]);
+                    stage[3 * lane + 1] = make_float4(o[1][1], o[1][2], o[2][0], o[2][1]);
+                    stage[3 * lane + 2] = make_float4(o[2][2], o[3][0], o[3][1], o[3][2]);
+                }
+                __syncwarp();
+                float4* dst = (a == 0 ? chol : color) + 3 * (size_t)qb;
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            float4* dst = (a == 0 ? chol : color) + 3 * (size_t)q;
-            dst[0] = make_float4(o[a][0][0], o[a][0][1], o[a][0][2], o[a][1][0]);
-            dst[1] = make_float4(o[a][1][1], o[a][1][2], o[a][2][0], o[a][2][1]);
-            dst[2] = make_float4(o[a][2][2], o[a][3][0], o[a][3][1], o[a][3][2]);
+                for (int i = 0; i < 3; ++i)
+                    if (lane + 32 * i < 3 * valid) dst[lane + 32 * i] = stage[lane + 32 * i];
+                __syncwarp();
+            }
         }
     }
 }
@@ -297,14 +272,19 @@ cudaError_t launch_vq_decode(const uint16_t* means16, const uint8_t* idx, const 
     auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
     if (out_stride_aos == 0 && n % 4 == 0 && a16(means16) && (reinterpret_cast<uintptr_t>(idx) & 3) == 0 &&
         a16(means) && a16(chol) && a16(color)) {
-        const size_t smem = (size_t)2 * stages * cb_size * sizeof(float4);
-        cudaError_t e = smem_optin(reinterpret_cast<const void*>(k_vq_decode4), (int)smem);
-        if (e != cudaSuccess) return e;
-        const int blocks = std::max(1, std::min((n / 4 + 255) / 256, sm_count() * 8));
-        k_vq_decode4<<<blocks, 256, smem, s>>>(reinterpret_cast<const uint2*>(means16), idx, cb, n, stages, cb_size,
+        auto go = [&](auto kern, int threads, int copies, int per_sm) {
+            const size_t smem = ((size_t)2 * stages * cb_size * copies + 96 * (threads / 32)) * sizeof(float4);
+            cudaError_t e = smem_optin(reinterpret_cast<const void*>(kern), (int)smem);
+            if (e != cudaSuccess) return e;
+            const int blocks = std::max(1, std::min((n / 4 + threads - 1) / threads, sm_count() * per_sm));
+            kern<<<blocks, threads, smem, s>>>(reinterpret_cast<const uint4*>(means16), idx, cb, n, stages, cb_size,
                                                reinterpret_cast<float4*>(means), reinterpret_cast<float4*>(chol),
-                                               reinterpret_cast<float4*>(color), device_status());
-        return cudaGetLastError();
+                                               reinterpret_cast<float4*>(color), copies,
+                                               (reinterpret_cast<uintptr_t>(means) & 31) == 0, device_status());
+            return cudaGetLastError();
+        };
+        if (stages == 2 && n >= kVqReplicated) return go(k_vq_decode4<2, 1024>, 1024, 8, 1);
+        return stages <= 2 ? go(k_vq_decode4<2, 256>, 256, 1, 8) : go(k_vq_decode4<8, 256>, 256, 1, 8);
     }
     const size_t smem = (size_t)2 * stages * cb_size * 3 * sizeof(float);
     {
