@@ -219,8 +219,10 @@ __global__ void __launch_bounds__(256) k_codec_decode(const uint16_t* __restrict
                                                       float* __restrict__ chol, float* __restrict__ color,
                                                       uint32_t* status) {
     extern __shared__ float scb[];  // [stages][size][3]
+    pdl_wait();
     for (int i = threadIdx.x; i < stages * size * 3; i += blockDim.x) scb[i] = cb[i];
     __syncthreads();
+    const bool two = stages <= 2;  // then one FP32 addition is the exact sum rounded once
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < n; g += gridDim.x * blockDim.x) {
         means[2 * (size_t)g] = __half2float(__ushort_as_half(means16[2 * (size_t)g]));
         means[2 * (size_t)g + 1] = __half2float(__ushort_as_half(means16[2 * (size_t)g + 1]));
@@ -229,6 +231,7 @@ __global__ void __launch_bounds__(256) k_codec_decode(const uint16_t* __restrict
         chol[3 * (size_t)g + 1] = __fadd_rn(__fmul_rn((float)q.y, gb.v[1]), gb.v[4]);
         chol[3 * (size_t)g + 2] = __fadd_rn(__fmul_rn((float)q.z, gb.v[2]), gb.v[5]);
         double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+        float f0 = 0.f, f1 = 0.f, f2 = 0.f;
         for (int m = 0; m < stages; ++m) {
             int j = idx[(size_t)m * n + g];
             if (j >= size) {  // index outside the codebook: skip the read
@@ -236,13 +239,19 @@ __global__ void __launch_bounds__(256) k_codec_decode(const uint16_t* __restrict
                 j = 0;
             }
             const float* e = scb + ((size_t)m * size + j) * 3;
-            s0 = __dadd_rn(s0, (double)e[0]);
-            s1 = __dadd_rn(s1, (double)e[1]);
-            s2 = __dadd_rn(s2, (double)e[2]);
+            if (two) {
+                f0 = __fadd_rn(f0, e[0]);
+                f1 = __fadd_rn(f1, e[1]);
+                f2 = __fadd_rn(f2, e[2]);
+            } else {
+                s0 = __dadd_rn(s0, (double)e[0]);
+                s1 = __dadd_rn(s1, (double)e[1]);
+                s2 = __dadd_rn(s2, (double)e[2]);
+            }
         }
-        color[3 * (size_t)g] = (float)s0;
-        color[3 * (size_t)g + 1] = (float)s1;
-        color[3 * (size_t)g + 2] = (float)s2;
+        color[3 * (size_t)g] = two ? f0 : (float)s0;
+        color[3 * (size_t)g + 1] = two ? f1 : (float)s1;
+        color[3 * (size_t)g + 2] = two ? f2 : (float)s2;
     }
 }
 
@@ -254,15 +263,10 @@ cudaError_t launch_codec_decode(const uint16_t* means16, const uint8_t* codes, c
     if (n <= 0) return cudaSuccess;
     GammaBeta gb;
     for (int i = 0; i < 6; ++i) gb.v[i] = gamma_beta[i];
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (nsm <= 0) nsm = 148;
-    const int blocks = std::max(1, std::min((n + 255) / 256, nsm * 4));
-    k_codec_decode<<<blocks, 256, (size_t)stages * size * 3 * sizeof(float), s>>>(
-        means16, reinterpret_cast<const uchar4*>(codes), gb, idx, cb, n, stages, size, means, chol, color,
-        device_status());
-    return cudaGetLastError();
+    const int blocks = std::max(1, std::min((n + 255) / 256, sm_count() * 4));
+    return launch_pdl(k_codec_decode, dim3(blocks), dim3(256), (size_t)stages * size * 3 * sizeof(float), s, means16,
+                      reinterpret_cast<const uchar4*>(codes), gb, idx, cb, n, stages, size, means, chol, color,
+                      device_status());
 }
 
 cudaError_t launch_vq_decode(const uint16_t* means16, const uint8_t* idx, const float* cb, int32_t n, int32_t stages,
