@@ -221,13 +221,11 @@ template <int T>
 __global__ void __launch_bounds__(kBwdThreads, 2) k_backward(
     const float4* __restrict__ rec_binned, const uint32_t* __restrict__ keys, const uint32_t* __restrict__ emit,
     const float* __restrict__ dl_tiled, Batch B, const int64_t* __restrict__ k_dev, int64_t capacity,
-    float4* __restrict__ partial, int32_t* __restrict__ step, uint32_t* __restrict__ status) {
+    float4* __restrict__ partial, AdamCfg adam, uint32_t* __restrict__ status) {
     constexpr int TF = tile_floats<T>();
     extern __shared__ float4 s_dyn[];
     pdl_wait();
-    // The optimiser's step counter, read by the kernels behind this one
-    // (counted here, the reduction's blocks need no last-block election).
-    if (step && blockIdx.x == 0 && threadIdx.x == 0) ++*step;
+    if (adam.step && blockIdx.x == 0 && threadIdx.x == 0) begin_update(adam);
     const int K = (int)min(*k_dev, capacity);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     BwdWarpSmem<T>& w = reinterpret_cast<BwdWarpSmem<T>*>(s_dyn)[wib];
@@ -490,15 +488,16 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(const float4* __restr
                                                 AdamCfg cfg, float* __restrict__ params, float* __restrict__ m,
                                                 float* __restrict__ v, float* __restrict__ grads_aos, Batch B,
                                                 const double* __restrict__ loss_tile, double* __restrict__ loss) {
-    __shared__ int s_step;
-    // Adam: 1/(1 - b1^t), 1/sqrt(1 - b2^t); Adan: 1/(1 - b1^t), 1/(1 - b2^t),
-    // 1/sqrt(1 - b3^t); [3] = learning-rate factor of the halving schedule.
-    __shared__ float s_bc[4];
     pdl_wait();
-    // The step counter's load (the backward has advanced it) is issued here
-    // and used after the partials are summed, so no load below waits for it.
-    int step = 0;
-    if (ADAM && threadIdx.x == 0) step = *cfg.step;
+    // The step and its bias corrections (see AdamCfg), loaded here and used
+    // after the partials are summed, so that nothing below waits for them.
+    int s_step = 0;
+    float s_bc[4] = {0.f, 0.f, 0.f, 0.f};
+    if (ADAM) {
+        s_step = *cfg.step;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s_bc[i] = cfg.bias[i];
+    }
     const int gblocks = (int)max(1, (n + kReduceThreads - 1) / kReduceThreads);
     // With loss_tile the first B.nimg blocks sum the images' squared errors
     // (first, so that they start in the first wave) and the Gaussian blocks
@@ -597,21 +596,6 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(const float4* __restr
                 __syncwarp();
             }
         }
-    }
-    if (ADAM) {
-        if (threadIdx.x == 0) {
-            s_step = step;
-            s_bc[0] = 1.f / (1.f - powf(cfg.beta1, (float)step));
-            if (cfg.optimizer == 1) {
-                s_bc[1] = 1.f / (1.f - powf(cfg.beta2, (float)step));
-                s_bc[2] = rsqrtf(1.f - powf(cfg.beta3, (float)step));
-            } else {
-                s_bc[1] = rsqrtf(1.f - powf(cfg.beta2, (float)step));
-                s_bc[2] = 0.f;
-            }
-            s_bc[3] = cfg.lr_halve_every > 0 ? ldexpf(1.f, -((step - 1) / cfg.lr_halve_every)) : 1.f;
-        }
-        __syncthreads();
     }
     // codec fine-tuning: this Gaussian's dL/dgamma, dL/dbeta terms, RVQ indices,
     // stage residuals and commitment term (zero when off or g >= n)
@@ -821,7 +805,7 @@ __global__ void __launch_bounds__(kCodecSumThreads) k_codec_update(CodecCfg Q, A
     const int v = blockIdx.x;
     const int MB = Q.stages * Q.size;
     const int step = *cfg.step;  // the backward has advanced it
-    float corr1 = 0.f, corr2 = 0.f, corr3 = 0.f;  // bias corrections
+    const float corr1 = cfg.bias[0], corr2 = cfg.bias[1], corr3 = cfg.bias[2];
     // What the last block needs besides the totals is fetched by every block of
     // a small codebook before its own sum (the last one is not known yet), so
     // that it does not wait for it afterwards.
@@ -829,12 +813,6 @@ __global__ void __launch_bounds__(kCodecSumThreads) k_codec_update(CodecCfg Q, A
     auto fetch = [&]() {
         for (int i = threadIdx.x; i < MB; i += blockDim.x) s_cnt[i] = Q.ema_count[i];
         for (int i = threadIdx.x; i < 3 * MB; i += blockDim.x) s_sum[i] = Q.ema_total[i];
-        if (threadIdx.x < 6) {
-            corr1 = 1.f / (1.f - powf(cfg.beta1, (float)step));
-            corr2 = cfg.optimizer == 1 ? 1.f / (1.f - powf(cfg.beta2, (float)step))
-                                       : rsqrtf(1.f - powf(cfg.beta2, (float)step));
-            corr3 = cfg.optimizer == 1 ? rsqrtf(1.f - powf(cfg.beta3, (float)step)) : 0.f;
-        }
     };
     if (early) fetch();
     double acc = 0.0;
@@ -886,7 +864,7 @@ __global__ void __launch_bounds__(kCodecSumThreads) k_codec_update(CodecCfg Q, A
     if (t < 6) {
         const float gr = (float)s_tot[t];
         Q.out[1 + t] = s_tot[t];
-        const float lr = cfg.lr[1] * (cfg.lr_halve_every > 0 ? ldexpf(1.f, -((step - 1) / cfg.lr_halve_every)) : 1.f);
+        const float lr = cfg.lr[1] * cfg.bias[3];
         float* p = Q.gb;
         float& m = p[6 + t];
         float& vv = p[12 + t];
@@ -938,7 +916,7 @@ int backward_blocks_per_sm() {
 template <int T>
 cudaError_t launch_backward_t(const float4* rec_binned, const uint32_t* keys, const uint32_t* emit,
                               const float* dl_tiled, const Batch& B, const int64_t* k_dev, int64_t capacity,
-                              float4* partial, uint32_t* status, cudaStream_t s, int32_t* step) {
+                              float4* partial, uint32_t* status, cudaStream_t s, const AdamCfg* adam) {
     cudaError_t e = smem_optin(reinterpret_cast<const void*>(k_backward<T>), (int)backward_smem<T>());
     if (e != cudaSuccess) return e;
     // persistent: one wave of resident blocks (no more than the tasks need)
@@ -946,19 +924,19 @@ cudaError_t launch_backward_t(const float4* rec_binned, const uint32_t* keys, co
     const int64_t full = (int64_t)sm_count() * backward_blocks_per_sm<T>();
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(full, (tasks + kBwdWarps - 1) / kBwdWarps));
     return launch_pdl(k_backward<T>, dim3(blocks), dim3(kBwdThreads), backward_smem<T>(), s, rec_binned, keys, emit,
-                      dl_tiled, B, k_dev, capacity, partial, step, status);
+                      dl_tiled, B, k_dev, capacity, partial, adam ? *adam : AdamCfg{}, status);
 }
 
 }  // namespace
 
 cudaError_t launch_backward(const float4* rec_binned, const uint32_t* keys, const uint32_t* emit,
                             const float* dl_tiled, const Batch& B, const int64_t* k_dev, int64_t capacity,
-                            float4* partial, uint32_t* status, cudaStream_t s, int32_t* step) {
+                            float4* partial, uint32_t* status, cudaStream_t s, const AdamCfg* adam) {
     if (capacity <= 0) return cudaSuccess;
     switch (B.tile) {
-        case 8: return launch_backward_t<8>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s, step);
-        case 16: return launch_backward_t<16>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s, step);
-        case 32: return launch_backward_t<32>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s, step);
+        case 8: return launch_backward_t<8>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s, adam);
+        case 16: return launch_backward_t<16>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s, adam);
+        case 32: return launch_backward_t<32>(rec_binned, keys, emit, dl_tiled, B, k_dev, capacity, partial, status, s, adam);
         default: return cudaErrorInvalidValue;
     }
 }

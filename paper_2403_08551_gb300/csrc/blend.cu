@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kBPix / PX) k_backward_blend(
     const float4* __restrict__ rec_binned, const uint32_t* __restrict__ ids, const float* __restrict__ o_eff,
     const int2* __restrict__ ranges, const int4* __restrict__ rect, const int64_t* __restrict__ pair_off, Batch B,
     const float* __restrict__ out, const int32_t* __restrict__ n_last, const float* __restrict__ dl_tiled,
-    int64_t capacity, float* __restrict__ partial, float* __restrict__ partial_o, float one, int32_t* __restrict__ step,
+    int64_t capacity, float* __restrict__ partial, float* __restrict__ partial_o, float one, AdamCfg adam,
     uint32_t* status) {
     constexpr int NT = kBPix / PX, NW = NT / 32;
     __shared__ float4 s_rec[kBChunk][2];
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kBPix / PX) k_backward_blend(
     __shared__ uint32_t s_has[NW];  // entries of the chunk with a sum from warp w
     __shared__ int s_max[NW];
     pdl_wait();
-    if (step && blockIdx.x == 0 && threadIdx.x == 0) ++*step;  // the optimiser's counter (see k_backward)
+    if (adam.step && blockIdx.x == 0 && threadIdx.x == 0) begin_update(adam);
     const int t = blockIdx.x;
     const TileGeo tg = tile_geo(B, ranges, t, status);
     const ImgDesc& d = tg.d;
@@ -493,12 +493,12 @@ cudaError_t launch_render_blend(const float4* rec_binned, const uint32_t* ids, c
 
 cudaError_t launch_backward_blend(const float4* rec_binned, const uint32_t* ids, const int2* ranges, const int4* rect,
                                   const int64_t* pair_off, const Batch& B, const float* out, const float* dl_tiled,
-                                  int64_t capacity, float4* partial, uint32_t* status, cudaStream_t s, int32_t* step) {
+                                  int64_t capacity, float4* partial, uint32_t* status, cudaStream_t s, const AdamCfg* adam) {
     if (B.total_tiles <= 0) return cudaSuccess;
     if (B.tile != kBT) return cudaErrorInvalidValue;
     return launch_pdl(k_backward_blend<kBlendBackwardPx>, dim3(B.total_tiles), dim3(kBPix / kBlendBackwardPx), 0, s,
                       rec_binned, ids, B.opac.o, ranges, rect, pair_off, B, out, B.opac.n_last, dl_tiled, capacity,
-                      reinterpret_cast<float*>(partial), B.opac.partial, 1.0f, step, status);
+                      reinterpret_cast<float*>(partial), B.opac.partial, 1.0f, adam ? *adam : AdamCfg{}, status);
 }
 
 }  // namespace gi

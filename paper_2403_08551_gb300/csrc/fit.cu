@@ -107,9 +107,9 @@ cudaError_t enqueue_step(gi_fit* f, cudaStream_t s) {
         NvtxRange r("gi:backward");
         e = f->B.opac.mode == 2
                 ? launch_backward_blend(f->rec_binned, f->ids, f->ranges, f->rect, f->pair_off, f->B, f->out,
-                                        f->dl_tiled, f->capacity, f->partial, device_status(), s, f->step)
+                                        f->dl_tiled, f->capacity, f->partial, device_status(), s, &f->adam)
                 : launch_backward(f->rec_binned, f->keys, f->emit, f->dl_tiled, f->B, f->k_dev, f->capacity,
-                                  f->partial, device_status(), s, f->step);
+                                  f->partial, device_status(), s, &f->adam);
     }
     if (e == cudaSuccess) e = mark(f, 4, s);
     if (e == cudaSuccess) {
@@ -279,7 +279,7 @@ gi_status gi_fit_create(const gi_fit_desc* d, gi_stream stream, gi_fit** out) {
         up256((size_t)f->capacity * 4), up256((size_t)f->capacity * 4),  // 15-16 keys ids
         up256((size_t)tiles * 8),                               // 17 ranges
         up256((size_t)d->n_images * 8),                         // 18 loss
-        256,                                                    // 19 step
+        256,                                                    // 19 step, bias corrections
         up256(probe.bytes),                                     // 20 bin ws
         d->optimizer == 1 ? up256((size_t)N * 32) : 0,          // 21 Adan n
         d->optimizer == 1 ? up256((size_t)N * 32) : 0,          // 22 Adan g_prev
@@ -350,6 +350,7 @@ gi_status gi_fit_create(const gi_fit_desc* d, gi_stream stream, gi_fit** out) {
     f->adam.beta2 = d->beta2;
     f->adam.eps = d->eps;
     f->adam.step = f->step;
+    f->adam.bias = reinterpret_cast<float*>(at(19) + 64);
     f->adam.optimizer = d->optimizer;
     f->adam.beta3 = d->beta3;
     f->adam.lr_halve_every = d->lr_halve_every;

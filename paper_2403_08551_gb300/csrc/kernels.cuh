@@ -114,6 +114,39 @@ cudaError_t launch_render(const float4* rec_binned, const int2* ranges, const Ba
                           double* loss_sum, double* loss_tile, uint32_t* status, cudaStream_t s,
                           const TileQueue* queue = nullptr);
 
+struct AdamCfg {
+    float lr[3];  // means, chol, color
+    float beta1, beta2, eps;
+    int32_t* step;  // device counter: the step of the update being made (the backward has advanced it)
+    float* bias;    // device [4], written by the backward for that step. Adam: 1/(1 - b1^t),
+                    // 1/sqrt(1 - b2^t); Adan: 1/(1 - b1^t), 1/(1 - b2^t), 1/sqrt(1 - b3^t);
+                    // [3] = learning-rate factor of the halving schedule
+    int32_t optimizer;       // 0: Adam; 1: Adan (beta1, beta2, beta3 decay m, v, n)
+    float beta3;             // Adan
+    int32_t lr_halve_every;  // every learning rate halves every this many steps; 0 = never
+    float* n;                // Adan: second moment of the extrapolated gradient [N][8]
+    float* g_prev;           // Adan: previous gradient [N][8]
+    int32_t param_mode;      // 1: params are the raw App. C.1 parameters (chain through the formation)
+    int32_t cov_mode;        // 1: covariance parameters are (theta, s1, s2) (chain dSigma -> theta, s1, s2)
+};
+
+// Start of a step's update (one thread, in the backward): advances the counter
+// and writes the step's bias corrections, so that no block of the reduction
+// computes or waits for them.
+__device__ __forceinline__ void begin_update(const AdamCfg& c) {
+    const int step = *c.step + 1;
+    *c.step = step;
+    c.bias[0] = 1.f / (1.f - powf(c.beta1, (float)step));
+    if (c.optimizer == 1) {
+        c.bias[1] = 1.f / (1.f - powf(c.beta2, (float)step));
+        c.bias[2] = rsqrtf(1.f - powf(c.beta3, (float)step));
+    } else {
+        c.bias[1] = rsqrtf(1.f - powf(c.beta2, (float)step));
+        c.bias[2] = 0.f;
+    }
+    c.bias[3] = c.lr_halve_every > 0 ? ldexpf(1.f, -((step - 1) / c.lr_halve_every)) : 1.f;
+}
+
 // Sorted alpha-blending render (Eq. 3-4) and its backward (blend.cu), tile 16
 // only; opacity, per-pixel walk lengths and the ninth per-pair sum live in
 // B.opac.
@@ -123,31 +156,19 @@ cudaError_t launch_render_blend(const float4* rec_binned, const uint32_t* ids, c
 cudaError_t launch_backward_blend(const float4* rec_binned, const uint32_t* ids, const int2* ranges, const int4* rect,
                                   const int64_t* pair_off, const Batch& B, const float* out, const float* dl_tiled,
                                   int64_t capacity, float4* partial, uint32_t* status, cudaStream_t s,
-                                  int32_t* step = nullptr);
+                                  const AdamCfg* adam = nullptr);
 
 // Backward: per-pair partial sums (8 floats per pair at its emission index
-// emit[k], written by the binning or by launch_emit_index). Both backwards
-// advance *step (nullable), the optimiser's step counter.
+// emit[k], written by the binning or by launch_emit_index). With adam
+// (fitting) both backwards begin the step's update (begin_update).
 cudaError_t launch_backward(const float4* rec_binned, const uint32_t* keys, const uint32_t* emit,
                             const float* dl_tiled, const Batch& B, const int64_t* k_dev, int64_t capacity,
-                            float4* partial, uint32_t* status, cudaStream_t s, int32_t* step = nullptr);
+                            float4* partial, uint32_t* status, cudaStream_t s, const AdamCfg* adam = nullptr);
 cudaError_t launch_emit_index(const uint32_t* keys, const uint32_t* ids, const int4* rect, const int64_t* pair_off,
                               const Batch& B, const int64_t* k_dev, int64_t capacity, uint32_t* emit,
                               uint32_t* status, cudaStream_t s);
 cudaError_t launch_pack_dl(const float* dl_hwc, const Batch& B, float* dl_tiled, cudaStream_t s);
 
-struct AdamCfg {
-    float lr[3];  // means, chol, color
-    float beta1, beta2, eps;
-    int32_t* step;  // device counter: the step of the update being made (the backward has advanced it)
-    int32_t optimizer;       // 0: Adam; 1: Adan (beta1, beta2, beta3 decay m, v, n)
-    float beta3;             // Adan
-    int32_t lr_halve_every;  // every learning rate halves every this many steps; 0 = never
-    float* n;                // Adan: second moment of the extrapolated gradient [N][8]
-    float* g_prev;           // Adan: previous gradient [N][8]
-    int32_t param_mode;      // 1: params are the raw App. C.1 parameters (chain through the formation)
-    int32_t cov_mode;        // 1: covariance parameters are (theta, s1, s2) (chain dSigma -> theta, s1, s2)
-};
 
 // Reduce partials per Gaussian, chain conic -> Cholesky; then either write
 // gradients (g_means/g_chol/g_color/g_conic, SoA, any may be null) or, when
