@@ -118,7 +118,16 @@ __device__ __forceinline__ int load_chunk(const int4* __restrict__ rect, const i
         cs.img[threadIdx.x] = im;
         cs.inv_w[threadIdx.x] = c > 0 ? __frcp_rn((float)(r.z - r.x)) : 0.f;
     }
-    const uint64_t incl = block_incl_scan<uint64_t>(((uint64_t)hi << 32) | (uint32_t)c, s_warp);
+    // Block scan with one barrier: every warp scans the warps' totals itself.
+    uint64_t incl = warp_incl_scan<uint64_t>(((uint64_t)hi << 32) | (uint32_t)c);
+    {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        const uint64_t w = warp_incl_scan<uint64_t>(lane < nw ? s_warp[lane] : 0ull);
+        const uint64_t below = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
+        if (warp > 0) incl += below;
+    }
     if (holds) cs.off[threadIdx.x + 1] = (int)(uint32_t)incl;
     if (hi_incl) *hi_incl = (uint32_t)(incl >> 32);
     if (threadIdx.x == 0) cs.off[0] = 0;
@@ -289,7 +298,7 @@ __global__ void __launch_bounds__(2 * CH) k_place(const int4* __restrict__ rect,
     constexpr int NG = CH / 32;  // lane groups
     constexpr int kRowLoads = (kCmMaxTiles + kPlaceThreads - 1) / kPlaceThreads;
     // [NG][total_tiles] lane masks, [total_tiles] P row (+ start), [total_tiles + 1] start
-    extern __shared__ uint32_t s_dyn[];
+    extern __shared__ __align__(16) uint32_t s_dyn[];
     __shared__ ChunkSmem<CH> cs;
     __shared__ float4 s_rec[CH][2];
     __shared__ uint64_t s_warp[32];
@@ -358,7 +367,10 @@ __global__ void __launch_bounds__(2 * CH) k_place(const int4* __restrict__ rect,
         s_rec[threadIdx.x][0] = rec[2 * (size_t)g];
         s_rec[threadIdx.x][1] = rec[2 * (size_t)g + 1];
     }
-    for (int i = threadIdx.x; i < NG * Tn; i += kPlaceThreads) s_m[i] = 0u;
+    for (int i = threadIdx.x; i < NG * Tn / 4; i += kPlaceThreads)  // NG is a multiple of 4
+        reinterpret_cast<uint4*>(s_m)[i] = make_uint4(0u, 0u, 0u, 0u);
+    pre = warp_sum<int64_t>(pre);
+    if ((threadIdx.x & 31) == 0) s_warp64[threadIdx.x >> 5] = pre;  // published by load_chunk's barriers
     uint32_t tsum = 0;
 #pragma unroll
     for (int i = 0; i < kTilesPerThread; ++i) tsum += tt[i];
@@ -379,7 +391,9 @@ __global__ void __launch_bounds__(2 * CH) k_place(const int4* __restrict__ rect,
         }
         if (threadIdx.x == kPlaceThreads - 1) s_start[Tn] = tincl;  // K
     }
-    pre = block_sum<int64_t>(pre, s_warp64);  // its barriers also publish the starts
+    pre = 0;
+#pragma unroll
+    for (int i = 0; i < kPlaceThreads / 32; ++i) pre += s_warp64[i];
     if (holds) {
         const int off = cs.off[threadIdx.x];
         if (g < B.total_gauss) pair_off[g] = pre + off;
