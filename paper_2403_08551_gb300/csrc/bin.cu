@@ -16,6 +16,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.cuh"
 
@@ -503,43 +504,42 @@ __global__ void __launch_bounds__(kProjBlock) k_emit(const int4* __restrict__ re
 
 // ---------------------------------------------------------------------------
 // One stable LSD radix pass (onesweep) over digits of up to 9 bits. Each
-// block takes a ticket, ranks its kSortTile keys per digit with warp-level
-// multi-split (items ordered by (warp, round, lane) = input order, so the
+// block takes a ticket, ranks its kSortThreads x ITEMS keys per digit with
+// warp-level multi-split (items ordered by (warp, round, lane) = input order, so the
 // ranking is stable), resolves its per-digit global offset with a decoupled
 // look-back over lower tickets (bounded spin), and scatters. A thread owns
 // digit threadIdx.x in the per-digit phases.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortThreads, 1) k_onesweep(
-    const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
-    uint32_t* __restrict__ vals_out, const int64_t* __restrict__ k_dev, int64_t capacity, int shift, int dbits,
-    const uint32_t* __restrict__ hist, uint32_t* __restrict__ lookback, uint32_t* __restrict__ ticket,
-    uint32_t* __restrict__ status) {
+struct SortSmem {
+    uint32_t s_wc[kSortThreads / 32][kMaxRadix];
+    uint32_t s_base[kMaxRadix];   // global position of the block's first key of each digit
+    uint32_t s_boff[kMaxRadix];   // block-local position of the first key of each digit
+    uint32_t s_warp[32];
+    uint32_t s_tot0;
+    uint32_t s_ticket;
+};
+
+template <int ITEMS>
+__device__ __forceinline__ void sort_block(int blk, int K, SortSmem& sm, const uint32_t* __restrict__ keys_in,
+                                           const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
+                                           uint32_t* __restrict__ vals_out, int shift, int dbits,
+                                           const uint32_t* __restrict__ hist, uint32_t* __restrict__ lookback,
+                                           uint32_t* __restrict__ status) {
     constexpr int NW = kSortThreads / 32;
     constexpr int DPT = kMaxRadix / kSortThreads;  // digits per thread in the per-digit phases
-    __shared__ uint32_t s_wc[NW][kMaxRadix];
-    __shared__ uint32_t s_base[kMaxRadix];   // global position of the block's first key of each digit
-    __shared__ uint32_t s_boff[kMaxRadix];   // block-local position of the first key of each digit
-    __shared__ uint32_t s_warp[32];
-    __shared__ uint32_t s_tot0;
-    __shared__ uint32_t s_ticket;
-    extern __shared__ uint32_t s_stage[];    // [kSortTile] keys, then [kSortTile] values, in digit order
-    pdl_wait();
-    const int K = (int)min(*k_dev, capacity);
-    if (threadIdx.x == 0) s_ticket = atomicAdd(ticket, 1u);
-    for (int i = threadIdx.x; i < NW * kMaxRadix; i += kSortThreads) (&s_wc[0][0])[i] = 0;
-    __syncthreads();
-    const int blk = (int)s_ticket;
-    const int64_t start = (int64_t)blk * kSortTile;
+    extern __shared__ uint32_t s_stage[];          // keys, then values, in digit order
+    constexpr int kTile = kSortThreads * ITEMS;
+    const int64_t start = (int64_t)blk * kTile;
     if (start >= K) return;
     const int radix = 1 << dbits;
     const uint32_t mask = (uint32_t)radix - 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    uint32_t key[kSortItems], val[kSortItems], lrank[kSortItems];
-    uint32_t dig[kSortItems];
+    uint32_t key[ITEMS], val[ITEMS], lrank[ITEMS];
+    uint32_t dig[ITEMS];
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t idx = start + warp * 32 * kSortItems + r * 32 + lane;
+    for (int r = 0; r < ITEMS; ++r) {
+        const int64_t idx = start + warp * 32 * ITEMS + r * 32 + lane;
         if (idx < K) {
             key[r] = keys_in[idx];
             val[r] = vals_in[idx];
@@ -550,10 +550,10 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_onesweep(
             dig[r] = kMaxRadix;  // no digit: not ranked, not stored
         }
     }
-    uint32_t* wc = s_wc[warp];
+    uint32_t* wc = sm.s_wc[warp];
     const uint32_t ltmask = lanemask_lt();
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
+    for (int r = 0; r < ITEMS; ++r) {
         const uint32_t dg = dig[r];
         // lanes with the same digit (keys past K carry kMaxRadix, a value no
         // digit has, and are grouped apart): one warp match
@@ -580,8 +580,8 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_onesweep(
         if (d < radix) {
 #pragma unroll
             for (int w = 0; w < NW; ++w) {
-                const uint32_t v = s_wc[w][d];
-                s_wc[w][d] = tot[q];
+                const uint32_t v = sm.s_wc[w][d];
+                sm.s_wc[w][d] = tot[q];
                 tot[q] += v;
             }
             st_relaxed_u32(lookback + (size_t)blk * kMaxRadix + d, (blk == 0 ? kFlagPre : kFlagAgg) | tot[q]);
@@ -600,17 +600,17 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_onesweep(
 #pragma unroll
                 for (int rep = 0; rep < kHistReplicas; ++rep) h += hist[rep * kMaxRadix + d];
             }
-            const uint32_t incl = block_incl_scan<uint32_t>(h, s_warp);  // ends with a barrier
+            const uint32_t incl = block_incl_scan<uint32_t>(h, sm.s_warp);  // ends with a barrier
             hex[q] = carry + incl - h;
-            if (threadIdx.x == kSortThreads - 1) s_tot0 = incl;
+            if (threadIdx.x == kSortThreads - 1) sm.s_tot0 = incl;
             __syncthreads();
-            carry += s_tot0;
+            carry += sm.s_tot0;
             __syncthreads();
-            const uint32_t lincl = block_incl_scan<uint32_t>(tot[q], s_warp);
-            if (d < radix) s_boff[d] = lcarry + lincl - tot[q];
-            if (threadIdx.x == kSortThreads - 1) s_tot0 = lincl;
+            const uint32_t lincl = block_incl_scan<uint32_t>(tot[q], sm.s_warp);
+            if (d < radix) sm.s_boff[d] = lcarry + lincl - tot[q];
+            if (threadIdx.x == kSortThreads - 1) sm.s_tot0 = lincl;
             __syncthreads();
-            lcarry += s_tot0;
+            lcarry += sm.s_tot0;
             __syncthreads();
         }
     }
@@ -652,32 +652,75 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_onesweep(
             }
             st_relaxed_u32(lookback + (size_t)blk * kMaxRadix + d, kFlagPre | ((excl + tot[q]) & kValMask));
         }
-        s_base[d] = hex[q] + excl;
+        sm.s_base[d] = hex[q] + excl;
     }
     // Stage the block's keys in digit order, then write each digit's run
     // with consecutive threads (coalesced stores).
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
+    for (int r = 0; r < ITEMS; ++r) {
         const uint32_t dg = dig[r];
         if (dg < kMaxRadix) {
-            const uint32_t li = s_boff[dg] + s_wc[warp][dg] + lrank[r];
+            const uint32_t li = sm.s_boff[dg] + sm.s_wc[warp][dg] + lrank[r];
             s_stage[li] = key[r];
-            s_stage[kSortTile + li] = val[r];
+            s_stage[kTile + li] = val[r];
         }
     }
     __syncthreads();
-    const int nvalid = (int)min((int64_t)kSortTile, (int64_t)K - start);
+    const int nvalid = (int)min((int64_t)kTile, (int64_t)K - start);
     for (int i = threadIdx.x; i < nvalid; i += kSortThreads) {
         const uint32_t kk = s_stage[i];
         const uint32_t dg = (kk >> shift) & mask;
-        const uint32_t pos = s_base[dg] + ((uint32_t)i - s_boff[dg]);
+        const uint32_t pos = sm.s_base[dg] + ((uint32_t)i - sm.s_boff[dg]);
         if (pos >= (uint32_t)K) {
             flag_error(status, kErrBounds);
             continue;
         }
         keys_out[pos] = kk;
-        vals_out[pos] = s_stage[kSortTile + i];
+        vals_out[pos] = s_stage[kTile + i];
     }
+}
+
+// Keys per thread for K keys. A block is latency-bound (ranking key by key,
+// barriers, look-back) and fills an SM's registers, so the sort takes as long as
+// its waves of kSortWave blocks: the fewest keys a thread that need one wave,
+// beyond that 12 if that needs no more waves than 16. Measured with 512 threads
+// at 16 / 12 / 8 / 4 keys (256 x 16 before): render of 1,000 x 1,422 / 51,000
+// Gaussians 67 / - / 59 / 56 us (65), 2040x1356 / 100,000 85 / - / 79.5 / 80.4
+// (90.7), 1,738 x 1,506 / 130,000 98 / 94.5 / 101 / 101 (104), 1,827 x 1,396 /
+// 200,000 124 / - / 130 / 132 (130); step of 1,633 x 1,443 / 104,000 at tile 8 316
+// / 310.5; 24 keys gain 5 us more there and cost 1 us everywhere else (spills).
+__device__ __forceinline__ int sort_items(int K) {
+    constexpr int w = kSortWave * kSortThreads;  // keys of one wave per item
+    if (K <= 4 * w) return 4;
+    if (K <= 8 * w) return 8;
+    if (K <= 12 * w) return 12;
+    if (K <= 16 * w) return 16;
+    return (K + 12 * w - 1) / (12 * w) > (K + 16 * w - 1) / (16 * w) ? 16 : 12;
+}
+
+__global__ void __launch_bounds__(kSortThreads, 1) k_onesweep(
+    const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
+    uint32_t* __restrict__ vals_out, const int64_t* __restrict__ k_dev, int64_t capacity, int shift, int dbits,
+    const uint32_t* __restrict__ hist, uint32_t* __restrict__ lookback, uint32_t* __restrict__ ticket,
+    uint32_t* __restrict__ status) {
+    __shared__ SortSmem sm;
+    pdl_wait();
+    const int K = (int)min(*k_dev, capacity);
+    const int items = sort_items(K);
+    // the blocks past the last key: out before they take a ticket
+    if ((int64_t)blockIdx.x * kSortThreads * items >= K) return;
+    if (threadIdx.x == 0) sm.s_ticket = atomicAdd(ticket, 1u);
+    for (int i = threadIdx.x; i < kSortThreads / 32 * kMaxRadix; i += kSortThreads) (&sm.s_wc[0][0])[i] = 0;
+    __syncthreads();
+    const int blk = (int)sm.s_ticket;
+    auto go = [&](auto c) {
+        sort_block<decltype(c)::value>(blk, K, sm, keys_in, vals_in, keys_out, vals_out, shift, dbits, hist, lookback,
+                                       status);
+    };
+    if (items == 16) go(std::integral_constant<int, 16>{});
+    else if (items == 12) go(std::integral_constant<int, 12>{});
+    else if (items == 8) go(std::integral_constant<int, 8>{});
+    else go(std::integral_constant<int, 4>{});
 }
 
 // ranges[t] = [first, last + 1) of key t in the sorted keys; with rec_binned,
@@ -752,6 +795,14 @@ __global__ void k_ranges(const uint32_t* __restrict__ keys, uint32_t* __restrict
     }
 }
 
+// Blocks that a sort of up to `capacity` keys may use (sort_items: never more
+// than the waves that 16 keys a thread take).
+int64_t sort_blocks(int64_t capacity) {
+    auto blocks = [&](int items) { return (capacity + kSortThreads * items - 1) / (kSortThreads * items); };
+    const int64_t wave16 = int64_t(kSortWave) * kSortThreads * 16;
+    return std::max<int64_t>(1, std::min<int64_t>(blocks(4), kSortWave * ((capacity + wave16 - 1) / wave16)));
+}
+
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
@@ -767,7 +818,7 @@ RadixPlan radix_plan(int total_tiles) {
 BinWs bin_ws_layout(void* base, int64_t n, int64_t capacity, int total_tiles, bool with_owner) {
     const RadixPlan rp = radix_plan(total_tiles);
     const int64_t nblk = std::max<int64_t>(1, (n + kProjBlock - 1) / kProjBlock);
-    const int64_t sblk = std::max<int64_t>(1, (capacity + kSortTile - 1) / kSortTile);
+    const int64_t sblk = sort_blocks(capacity);
     const int chunk = cm_chunk(n);
     const int64_t nchunks = std::max<int64_t>(1, (n + chunk - 1) / chunk);
     const int64_t cap = std::max<int64_t>(1, capacity);
@@ -823,7 +874,7 @@ cudaError_t launch_bin(const int4* rect, const int32_t* cnt, const float4* rec, 
     const RadixPlan rp = radix_plan(B.total_tiles);
     const int n = B.total_gauss;
     const int nblk = std::max(1, (n + kProjBlock - 1) / kProjBlock);
-    const int64_t sblk = std::max<int64_t>(1, (capacity + kSortTile - 1) / kSortTile);
+    const int64_t sblk = sort_blocks(capacity);
     if (!blk_sum_ready) {
         ZeroJob zj{};
         zj.p[0] = ws.zero;

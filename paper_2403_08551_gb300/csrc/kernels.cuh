@@ -32,18 +32,13 @@ struct RadixPlan {
 RadixPlan radix_plan(int total_tiles);
 
 constexpr int kProjBlock = 256;        // Gaussians per projection / emit block
-// 8,192 keys a block: half the blocks and so half the look-back rounds of 256
-// threads, and at 1 M pairs every SM has at most one (step 308.2 -> 305.8 us at
-// 2040x1356 / 200,000, 731.5 -> 724.2 us on 16 uneven images; 512 x 8: 307.5,
-// 726.9; 1024 x 8: 307.8, 729.3; 512 x 12: 314.4, 728.4).
 constexpr int kSortThreads = 512;      // threads per onesweep block
-constexpr int kSortItems = 16;         // keys per thread
+constexpr int kSortWave = 152;         // onesweep blocks that run at the same time (one per SM)
 constexpr int kMaxDigitBits = 9;       // radix digits of at most 9 bits (512 buckets)
 constexpr int kMaxRadix = 1 << kMaxDigitBits;
 constexpr int kMaxPasses = 4;          // 31-bit keys at most
 constexpr int kHistReplicas = 8;       // copies of each pass's digit histogram (spread the emit's atomics)
-constexpr int kSortTile = kSortThreads * kSortItems;  // keys per onesweep block
-constexpr int kSortStageBytes = kSortTile * 8;          // keys + values staged in digit order
+constexpr int kSortStageBytes = kSortThreads * 16 * 8;  // keys + values of a block staged in digit order
 
 // Count-matrix binning (bin_cm.cu): chunks of cm_chunk(n) Gaussians; used when
 // the batch has at most kCmMaxTiles tiles and 128-Gaussian rows x tiles <=
