@@ -4,7 +4,7 @@
 // The result equals the sum evaluated exactly and rounded once to FP32: for
 // M <= 2 a single FP32 addition already is that (rounding a double-precision
 // sum of two floats to float is innocuous since 53 >= 2*24 + 2); for M > 2
-// the stages are accumulated in FP64 and rounded once.
+// it is what an FP64 sum in stage order, rounded once, gives (RowSum).
 #include <algorithm>
 
 #include <cuda_fp16.h>
@@ -13,6 +13,30 @@
 
 namespace gi {
 namespace {
+
+// The FP64 sum of up to eight floats rounded to FP32, on the FP32 units (with
+// FP64 a three-stage decode took five times a two-stage one): s + e is the
+// running sum and the errors of its additions (Knuth, TAOCP 2, 4.2.2), p the sum
+// of the magnitudes, q the smallest but for zeros. If q >= 2^-22 p, all terms are
+// multiples of 2^-45 p: then e (below 2^-21 p) and the FP64 sum are both exact, so
+// that s + e rounds as it does. Otherwise (terms of very different size,
+// infinities, NaN) get() is false and the caller sums in FP64. Three stages,
+// 64 entries: 1 M Gaussians 88 -> 16.5 us, 3.2 M x 256 entries 256 -> 43.6 us (what
+// bounds it there is the codebook rows' bank conflicts).
+struct RowSum {
+    float s = 0.f, e = 0.f, p = 0.f, q = 3.402823466e38f;
+    __device__ __forceinline__ void add(float x) {
+        const float t = __fadd_rn(s, x), v = __fsub_rn(t, s);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(x, v)));
+        s = t;
+        p = __fadd_rn(p, fabsf(x));
+        if (x != 0.f) q = fminf(q, fabsf(x));
+    }
+    __device__ __forceinline__ bool get(float& r) const {
+        r = __fadd_rn(s, e);
+        return q >= __fmul_rn(p, 0x1p-22f);
+    }
+};
 
 __global__ void __launch_bounds__(256) k_vq_decode(const uint16_t* __restrict__ means16,
                                                    const uint8_t* __restrict__ idx, const float* __restrict__ cb,
@@ -43,7 +67,7 @@ __global__ void __launch_bounds__(256) k_vq_decode(const uint16_t* __restrict__ 
                 }
                 o[a][0] = acc[0]; o[a][1] = acc[1]; o[a][2] = acc[2];
             } else {
-                double acc[3] = {0.0, 0.0, 0.0};
+                RowSum sum[3];
                 for (int s = 0; s < stages; ++s) {
                     int i = idx[((size_t)a * stages + s) * n + g];
                     if (i >= cbs) {
@@ -51,11 +75,20 @@ __global__ void __launch_bounds__(256) k_vq_decode(const uint16_t* __restrict__ 
                         i = 0;
                     }
                     const float* row = scb + (((size_t)a * stages + s) * cbs + i) * 3;
-                    acc[0] += (double)row[0];
-                    acc[1] += (double)row[1];
-                    acc[2] += (double)row[2];
+                    for (int c = 0; c < 3; ++c) sum[c].add(row[c]);
                 }
-                o[a][0] = (float)acc[0]; o[a][1] = (float)acc[1]; o[a][2] = (float)acc[2];
+                bool ok = true;
+                for (int c = 0; c < 3; ++c) ok &= sum[c].get(o[a][c]);
+                if (!ok) {
+                    double acc[3] = {0.0, 0.0, 0.0};
+                    for (int s = 0; s < stages; ++s) {
+                        int i = idx[((size_t)a * stages + s) * n + g];
+                        if (i >= cbs) i = 0;
+                        const float* row = scb + (((size_t)a * stages + s) * cbs + i) * 3;
+                        for (int c = 0; c < 3; ++c) acc[c] += (double)row[c];
+                    }
+                    for (int c = 0; c < 3; ++c) o[a][c] = (float)acc[c];
+                }
             }
         }
         if (aos_stride == 8) {
@@ -86,38 +119,83 @@ constexpr int kVqQuads = 2;  // quads per thread and round of the fast path
 // stage gains nothing (25 us either way).
 constexpr int kVqReplicated = 1200000;
 
+// RowSum's FP64 case for Gaussian j of a quad. Not inlined: the compiler would
+// otherwise run it for every value and choose.
+template <int MAXS>
+struct VqWords {
+    uint32_t w[MAXS];
+};
+template <int MAXS>
+__device__ __noinline__ float3 row_sum_fp64(VqWords<MAXS> ws, int j, const float4* rows, int copies, int stages,
+                                            int cbs) {
+    double d[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int st = 0; st < MAXS; ++st) {
+        if (st < stages) {
+            int i = (ws.w[st] >> (8 * j)) & 0xff;
+            if (i >= cbs) i = 0;
+            const float4 r = rows[(st * cbs + i) * copies];
+            d[0] += (double)r.x;
+            d[1] += (double)r.y;
+            d[2] += (double)r.z;
+        }
+    }
+    return make_float3((float)d[0], (float)d[1], (float)d[2]);
+}
+
 // The decoded attribute a (0: Cholesky vector, 1: colour) of a quad from its
 // index words w[stage] and the padded codebook rows: up to two stages as FP32
-// sums (exact), more in FP64, rounded once.
+// sums (exact), more as RowSum.
 template <int MAXS>
 __device__ __forceinline__ void vq_quad(const uint32_t (&w)[MAXS], const float4* rows, int copies, int stages,
                                         int cbs, float (&o)[4][3], uint32_t* status) {
+    auto row = [&](int st, int j) {
+        int i = (w[st] >> (8 * j)) & 0xff;
+        if (i >= cbs) {  // index outside the codebook: skip the read
+            flag_error(status, kErrBounds);
+            i = 0;
+        }
+        return rows[(st * cbs + i) * copies];
+    };
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        float f[3] = {0.f, 0.f, 0.f};
-        double d[3] = {0.0, 0.0, 0.0};
+        if constexpr (MAXS <= 2) {
+            float f[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-        for (int st = 0; st < MAXS; ++st) {
-            if (st < stages) {
-                int i = (w[st] >> (8 * j)) & 0xff;
-                if (i >= cbs) {  // index outside the codebook: skip the read
-                    flag_error(status, kErrBounds);
-                    i = 0;
-                }
-                const float4 r = rows[(st * cbs + i) * copies];
-                if (MAXS <= 2) {
+            for (int st = 0; st < MAXS; ++st) {
+                if (st < stages) {
+                    const float4 r = row(st, j);
                     f[0] = __fadd_rn(f[0], r.x);
                     f[1] = __fadd_rn(f[1], r.y);
                     f[2] = __fadd_rn(f[2], r.z);
-                } else {
-                    d[0] += (double)r.x;
-                    d[1] += (double)r.y;
-                    d[2] += (double)r.z;
                 }
             }
-        }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) o[j][c] = MAXS <= 2 ? f[c] : (float)d[c];
+            for (int c = 0; c < 3; ++c) o[j][c] = f[c];
+        } else {
+            RowSum sum[3];
+#pragma unroll
+            for (int st = 0; st < MAXS; ++st) {
+                if (MAXS == 3 || st < stages) {
+                    const float4 r = row(st, j);
+                    sum[0].add(r.x);
+                    sum[1].add(r.y);
+                    sum[2].add(r.z);
+                }
+            }
+            bool ok = true;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) ok &= sum[c].get(o[j][c]);
+            if (!ok) {
+                VqWords<MAXS> ws;
+#pragma unroll
+                for (int st = 0; st < MAXS; ++st) ws.w[st] = w[st];
+                const float3 d = row_sum_fp64<MAXS>(ws, j, rows, copies, MAXS == 3 ? 3 : stages, cbs);
+                o[j][0] = d.x;
+                o[j][1] = d.y;
+                o[j][2] = d.z;
+            }
+        }
     }
 }
 
@@ -288,7 +366,8 @@ cudaError_t launch_vq_decode(const uint16_t* means16, const uint8_t* idx, const 
             return cudaGetLastError();
         };
         if (stages == 2 && n >= kVqReplicated) return go(k_vq_decode4<2, 1024>, 1024, 8, 1);
-        return stages <= 2 ? go(k_vq_decode4<2, 256>, 256, 1, 8) : go(k_vq_decode4<8, 256>, 256, 1, 8);
+        if (stages <= 2) return go(k_vq_decode4<2, 256>, 256, 1, 8);
+        return stages == 3 ? go(k_vq_decode4<3, 256>, 256, 1, 8) : go(k_vq_decode4<8, 256>, 256, 1, 8);
     }
     const size_t smem = (size_t)2 * stages * cb_size * 3 * sizeof(float);
     {
