@@ -103,23 +103,16 @@ __device__ __forceinline__ void render_tile(int t, uint32_t& phase, const RSmem<
     // now (cp.async): their latency, long when the target is read from host
     // memory over the host link, overlaps the accumulation below.
     if (target) {
-        const float* t0 = target + 3 * (d.pix_base + (int64_t)y0 * d.W + x0);
-        const bool whole = x0 + T <= d.W && y0 + T <= d.H;
-        if (whole && d.W % 4 == 0 && (reinterpret_cast<uintptr_t>(t0) & 15) == 0) {
-            // whole tile, every row of it 16-byte aligned: 3 T / 4 copies a row
-            for (int q = threadIdx.x; q < 3 * NPIX / 4; q += NT) {
-                const int yy = q / (3 * T / 4), c = q % (3 * T / 4);
-                cp_async16(&s_tgt[4 * q], t0 + (int64_t)yy * 3 * d.W + 4 * c);
-            }
-        } else {
-            for (int p = threadIdx.x; p < NPIX; p += NT) {
-                const int x = x0 + p % T, y = y0 + p / T;
-                if (x < d.W && y < d.H) {
-                    const float* src = target + 3 * (d.pix_base + (int64_t)y * d.W + x);
-                    cp_async4(&s_tgt[3 * p], src);
-                    cp_async4(&s_tgt[3 * p + 1], src + 1);
-                    cp_async4(&s_tgt[3 * p + 2], src + 2);
-                }
+        // Through L1 (cp.async.ca): with 16-byte copies past it (.cg) a step on a
+        // target in host memory takes 143 us instead of 117 (768x512 / 70,000), and
+        // one in device memory is no faster.
+        for (int p = threadIdx.x; p < NPIX; p += NT) {
+            const int x = x0 + p % T, y = y0 + p / T;
+            if (x < d.W && y < d.H) {
+                const float* src = target + 3 * (d.pix_base + (int64_t)y * d.W + x);
+                cp_async4(&s_tgt[3 * p], src);
+                cp_async4(&s_tgt[3 * p + 1], src + 1);
+                cp_async4(&s_tgt[3 * p + 2], src + 2);
             }
         }
     }
@@ -189,9 +182,8 @@ __device__ __forceinline__ void render_tile(int t, uint32_t& phase, const RSmem<
     // pixels permuted by part_at so that the eight lanes of a 16-byte store
     // phase (two row blocks of four columns) fall on all 32 banks. With scalar
     // stores the groups' equal offsets made eight-way conflicts: at short
-    // lists that, and the target's 4-byte copies above, was the largest
-    // per-tile cost (render stage, 93 pairs a tile, 2040x1356 / 200k: 87.7 ->
-    // 85.7 us; 225 pairs a tile: unchanged).
+    // lists that was the largest per-tile cost (render stage, 93 pairs a tile,
+    // 2040x1356 / 200k: 87.7 -> 85.7 us; 225 pairs a tile: unchanged).
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
         if constexpr (PX % 4 == 0) {
