@@ -43,7 +43,7 @@ LR = (1e-3, 1e-2, 1e-2)
 FWD_FLOP_PER_EVAL = 13   # sigma 7 + 3 FFMA (accumulate)
 BWD_FLOP_PER_EVAL = 24   # sigma 7 + 3 FFMA (dL/dc') + FMUL + 2 FFMA (<G, c'>) + FMUL (e) + FADD + FMUL + FADD + FFMA (moments)
 # DRAM bytes (read + write) per launch of the ALU-bound kernels at this
-# workload, from one ncu --set full capture of the current kernels
+# workload, from one ncu --set full capture of each
 # (profiles/k_backward_c1_768x512_70k.md, profiles/k_render_c1_768x512_70k.md).
 NCU_TRAFFIC_BYTES = {"k_backward": 20.628e6, "k_render": 16.187e6}
 # SFU_LANES: ex2 results per clock per SM as measured by gi_alu_peaks on GB300
@@ -77,14 +77,15 @@ def pack(w):
 
 
 def binning_launches(n, W, H, T):
-    """Kernels the fit step's binning launches: 2 for the count-matrix path (at
-    most 2048 tiles and 128-Gaussian chunks x tiles <= 2^20; the projection
-    writes the count rows), else emit + one onesweep per LSD pass (digits of
-    at most 9 bits) + ranges."""
+    """Kernels the fit step's binning launches. The count-matrix path (at most
+    2048 tiles and 128-Gaussian rows x tiles <= 2^20; the projection writes the
+    counts): column scan and placement, the placement alone for at most 8,192
+    counts (chunks of 128 Gaussians up to 8,192 of them, else 256). Otherwise
+    emit + one onesweep per LSD pass (digits of at most 9 bits) + ranges."""
     tiles = ((W + T - 1) // T) * ((H + T - 1) // T)
-    chunks = max(1, (n + 127) // 128)
-    if tiles <= 2048 and chunks * tiles <= (1 << 20):
-        return 2
+    if tiles <= 2048 and max(1, (n + 127) // 128) * tiles <= (1 << 20):
+        chunk = 128 if n <= 8192 else 256
+        return 1 if max(1, (n + chunk - 1) // chunk) * tiles <= 8192 else 2
     bits = max(1, math.ceil(math.log2(max(tiles, 2))))
     return 2 + (bits + 8) // 9
 
