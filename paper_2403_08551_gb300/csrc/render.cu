@@ -301,9 +301,12 @@ __device__ __forceinline__ void render_tile(int t, uint32_t& phase, const RSmem<
 // lets the compiler use the registers it wants (98 instead of 80 at split 4,
 // where shared memory bounds the residency anyway): render stage 85.7 -> 79.5
 // us at 2040x1356 / 200k with the wide partial stores below (87.7 before both),
-// 178 -> 172 us on 16 uneven images.
+// 178 -> 172 us on 16 uneven images. Not at tile 32, whose blocks would take 68
+// registers instead of 48 and fewer would be resident: with a crowd of tiles in
+// one corner the step takes 304 to 342 us without the bound and 324 to 336 with
+// it, by where the corner lies (1120x1109 / 108k; 316 to 352 before both).
 template <class Cfg>
-__global__ void __launch_bounds__(Cfg::kThreads, 1) k_render(const float4* __restrict__ rec_binned,
+__global__ void __launch_bounds__(Cfg::kThreads, Cfg::T == 32 ? 0 : 1) k_render(const float4* __restrict__ rec_binned,
                                                           const int2* __restrict__ ranges, Batch B,
                                                           const float* __restrict__ target, float* __restrict__ out,
                                                           float* __restrict__ dl_hwc, float* __restrict__ dl_tiled,
