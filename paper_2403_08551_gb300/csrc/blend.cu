@@ -24,6 +24,8 @@
 // (colour, and e~ (dx, dy, dx^2, dx dy, dy^2) with e~ = -dL/dsigma) plus a
 // ninth for the opacity, at the pair's emission index; the per-Gaussian
 // reduction is then shared with the accumulated path. Deterministic.
+#include <type_traits>
+
 #include "kernels.cuh"
 
 namespace gi {
@@ -345,6 +347,7 @@ __global__ void __launch_bounds__(kBPix / PX) k_backward_blend(
     auto put = [](float2& v, int i, float f) { (i % 2 ? v.y : v.x) = f; };
     auto get = [](const float2& v, int i) { return i % 2 ? v.y : v.x; };
     int mine = 0;
+    bool finite = true;
 #pragma unroll
     for (int i = 0; i < PX; ++i) {
         const int q = tid + NT * i, h = i / 2;
@@ -368,7 +371,9 @@ __global__ void __launch_bounds__(kBPix / PX) k_backward_blend(
         P0[h] = P1[h] = P2[h] = make_float2(0.f, 0.f);
         Tr[h] = make_float2(1.f, 1.f);
         mine = max(mine, nl[i]);
+        finite = finite && isfinite(dt[q]) && isfinite(dt[kBPix + q]) && isfinite(dt[2 * kBPix + q]);
     }
+    const bool all_finite = __all_sync(0xffffffffu, finite);
     const int wmax = __reduce_max_sync(0xffffffffu, mine);  // entries this warp walks
     if (lane == 0) s_max[warp] = wmax;
     __syncthreads();
@@ -390,65 +395,77 @@ __global__ void __launch_bounds__(kBPix / PX) k_backward_blend(
         __syncthreads();
         const int walk = min(n, wmax - (base - tg.b));
         uint32_t has = 0;
-        for (int j = 0; j < walk; ++j) {
-            const float4 r0 = s_rec[j][0], r1 = s_rec[j][1];
-            const float o = s_o[j];
-            const int pos = base - tg.b + j;
-            const float dx = __fsub_rn(cx, r0.x);
-            const float z1 = __fmul_rn(r0.z, dx);
-            const float z1s = __fmul_rn(z1, z1), tt = __fmul_rn(r0.w, dx);
-            const float2 c0 = make_float2(r1.y, r1.y), c1 = make_float2(r1.z, r1.z), c2 = make_float2(r1.w, r1.w);
-            const float2 m1 = make_float2(-1.f, -1.f);
-            float v[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            // Branch-free, two pixels at a time: a pixel that skips the entry
-            // (or stopped before it) adds zeros and keeps its state; a pair of
-            // rows none of whose pixels sees the entry is passed over.
+        // A pixel that skips an entry adds dL/dC * 0, which is zero only while
+        // dL/dC is finite: with a non-finite target pixel in the warp's rows the
+        // skipped products are left out (as a branch in every walk it would cost
+        // issue slots; here the usual walk is unchanged).
+        auto walk_entries = [&](auto skip_zeros) {
+            for (int j = 0; j < walk; ++j) {
+                const float4 r0 = s_rec[j][0], r1 = s_rec[j][1];
+                const float o = s_o[j];
+                const int pos = base - tg.b + j;
+                const float dx = __fsub_rn(cx, r0.x);
+                const float z1 = __fmul_rn(r0.z, dx);
+                const float z1s = __fmul_rn(z1, z1), tt = __fmul_rn(r0.w, dx);
+                const float2 c0 = make_float2(r1.y, r1.y), c1 = make_float2(r1.z, r1.z), c2 = make_float2(r1.w, r1.w);
+                const float2 m1 = make_float2(-1.f, -1.f);
+                float v[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                // Branch-free, two pixels at a time: a pixel that skips the entry
+                // (or stopped before it) adds zeros and keeps its state; a pair of
+                // rows none of whose pixels sees the entry is passed over.
 #pragma unroll
-            for (int h = 0; h < PX / 2; ++h) {
-                const float2 dy = __fadd2_rn(cy[h], make_float2(-r0.y, -r0.y));
-                const float2 w = blend_w2(r1.x, z1s, tt, dy, one);
-                float2 a = __fmul2_rn(make_float2(o, o), w);
-                const bool u0 = !(a.x < kBlendAlphaMin) && pos < nl[2 * h];
-                const bool u1 = !(a.y < kBlendAlphaMin) && pos < nl[2 * h + 1];
-                if (!__any_sync(0xffffffffu, u0 || u1)) continue;
-                has |= 1u << j;
-                const bool f0 = u0 && !(a.x > kBlendAlphaMax), f1 = u1 && !(a.y > kBlendAlphaMax);  // not clamped
-                a = make_float2(fminf(a.x, kBlendAlphaMax), fminf(a.y, kBlendAlphaMax));
-                float2 at = __fmul2_rn(a, Tr[h]);
-                at = make_float2(u0 ? at.x : 0.f, u1 ? at.y : 0.f);
-                P0[h] = add_product(__fmul2_rn(c0, at), P0[h], one);  // as the forward pass rounds them
-                P1[h] = add_product(__fmul2_rn(c1, at), P1[h], one);
-                P2[h] = add_product(__fmul2_rn(c2, at), P2[h], one);
-                const float2 keep = __fadd2_rn(make_float2(1.f, 1.f), make_float2(-a.x, -a.y));
-                const float2 ninv = make_float2(-__fdividef(1.f, keep.x), -__fdividef(1.f, keep.y));
-                // dL/dalpha = sum_ch dL/dC (c T - (C - P) / (1 - alpha))
-                const float2 A = __ffma2_rn(c0, Tr[h], __fmul2_rn(__ffma2_rn(P0[h], m1, Cf0[h]), ninv));
-                const float2 Bb = __ffma2_rn(c1, Tr[h], __fmul2_rn(__ffma2_rn(P1[h], m1, Cf1[h]), ninv));
-                const float2 C = __ffma2_rn(c2, Tr[h], __fmul2_rn(__ffma2_rn(P2[h], m1, Cf2[h]), ninv));
-                float2 dla = __ffma2_rn(g2[h], C, __ffma2_rn(g0[h], A, __fmul2_rn(g1[h], Bb)));
-                dla = make_float2(f0 ? dla.x : 0.f, f1 ? dla.y : 0.f);
-                const float2 ee = __fmul2_rn(dla, a);  // -dL/dsigma
-                const float2 ex = __fmul2_rn(ee, make_float2(dx, dx)), ey = __fmul2_rn(ee, dy);
+                for (int h = 0; h < PX / 2; ++h) {
+                    const float2 dy = __fadd2_rn(cy[h], make_float2(-r0.y, -r0.y));
+                    const float2 w = blend_w2(r1.x, z1s, tt, dy, one);
+                    float2 a = __fmul2_rn(make_float2(o, o), w);
+                    const bool u0 = !(a.x < kBlendAlphaMin) && pos < nl[2 * h];
+                    const bool u1 = !(a.y < kBlendAlphaMin) && pos < nl[2 * h + 1];
+                    if (!__any_sync(0xffffffffu, u0 || u1)) continue;
+                    has |= 1u << j;
+                    const bool f0 = u0 && !(a.x > kBlendAlphaMax), f1 = u1 && !(a.y > kBlendAlphaMax);  // not clamped
+                    a = make_float2(fminf(a.x, kBlendAlphaMax), fminf(a.y, kBlendAlphaMax));
+                    float2 at = __fmul2_rn(a, Tr[h]);
+                    at = make_float2(u0 ? at.x : 0.f, u1 ? at.y : 0.f);
+                    P0[h] = add_product(__fmul2_rn(c0, at), P0[h], one);  // as the forward pass rounds them
+                    P1[h] = add_product(__fmul2_rn(c1, at), P1[h], one);
+                    P2[h] = add_product(__fmul2_rn(c2, at), P2[h], one);
+                    const float2 keep = __fadd2_rn(make_float2(1.f, 1.f), make_float2(-a.x, -a.y));
+                    const float2 ninv = make_float2(-__fdividef(1.f, keep.x), -__fdividef(1.f, keep.y));
+                    // dL/dalpha = sum_ch dL/dC (c T - (C - P) / (1 - alpha))
+                    const float2 A = __ffma2_rn(c0, Tr[h], __fmul2_rn(__ffma2_rn(P0[h], m1, Cf0[h]), ninv));
+                    const float2 Bb = __ffma2_rn(c1, Tr[h], __fmul2_rn(__ffma2_rn(P1[h], m1, Cf1[h]), ninv));
+                    const float2 C = __ffma2_rn(c2, Tr[h], __fmul2_rn(__ffma2_rn(P2[h], m1, Cf2[h]), ninv));
+                    float2 dla = __ffma2_rn(g2[h], C, __ffma2_rn(g0[h], A, __fmul2_rn(g1[h], Bb)));
+                    dla = make_float2(f0 ? dla.x : 0.f, f1 ? dla.y : 0.f);
+                    const float2 ee = __fmul2_rn(dla, a);  // -dL/dsigma
+                    const float2 ex = __fmul2_rn(ee, make_float2(dx, dx)), ey = __fmul2_rn(ee, dy);
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {  // one pixel after the other: the order of the sums
-                    v[0] = fmaf(get(g0[h], i), get(at, i), v[0]);
-                    v[1] = fmaf(get(g1[h], i), get(at, i), v[1]);
-                    v[2] = fmaf(get(g2[h], i), get(at, i), v[2]);
-                    v[3] = __fadd_rn(v[3], get(ex, i));
-                    v[4] = __fadd_rn(v[4], get(ey, i));
-                    v[5] = fmaf(get(ex, i), dx, v[5]);
-                    v[6] = fmaf(get(ex, i), get(dy, i), v[6]);
-                    v[7] = fmaf(get(ey, i), get(dy, i), v[7]);
-                    v[8] = fmaf(get(dla, i), get(w, i), v[8]);
+                    for (int i = 0; i < 2; ++i) {  // one pixel after the other: the order of the sums
+                        if (decltype(skip_zeros)::value ? (i ? u1 : u0) : true) {
+                            v[0] = fmaf(get(g0[h], i), get(at, i), v[0]);
+                            v[1] = fmaf(get(g1[h], i), get(at, i), v[1]);
+                            v[2] = fmaf(get(g2[h], i), get(at, i), v[2]);
+                        }
+                        v[3] = __fadd_rn(v[3], get(ex, i));
+                        v[4] = __fadd_rn(v[4], get(ey, i));
+                        v[5] = fmaf(get(ex, i), dx, v[5]);
+                        v[6] = fmaf(get(ex, i), get(dy, i), v[6]);
+                        v[7] = fmaf(get(ey, i), get(dy, i), v[7]);
+                        v[8] = fmaf(get(dla, i), get(w, i), v[8]);
+                    }
+                    const float2 Tn = __fmul2_rn(Tr[h], keep);
+                    Tr[h] = make_float2(u0 ? Tn.x : Tr[h].x, u1 ? Tn.y : Tr[h].y);
                 }
-                const float2 Tn = __fmul2_rn(Tr[h], keep);
-                Tr[h] = make_float2(u0 ? Tn.x : Tr[h].x, u1 ? Tn.y : Tr[h].y);
+                if (!((has >> j) & 1u)) continue;
+                const float s8 = warp_sum(v[8]), sum = warp_reduce_scatter8(v, lane);
+                if ((lane & 3) == 0) s_red[j][warp][lane >> 2] = sum;
+                if (lane == 1) s_red[j][warp][8] = s8;
             }
-            if (!((has >> j) & 1u)) continue;
-            const float s8 = warp_sum(v[8]), sum = warp_reduce_scatter8(v, lane);
-            if ((lane & 3) == 0) s_red[j][warp][lane >> 2] = sum;
-            if (lane == 1) s_red[j][warp][8] = s8;
-        }
+        };
+        if (all_finite)
+            walk_entries(std::false_type{});
+        else
+            walk_entries(std::true_type{});
         if (lane == 0) s_has[warp] = has;
         __syncthreads();
         for (int i = tid; i < n * 9; i += NT) {
