@@ -196,11 +196,12 @@ GI_API gi_status gi_render_pass(const float* means, const float* chol, const flo
  * pass, with everything the backward needs kept in one caller-owned buffer.
  *   state, state_bytes  *forward_bytes of gi_rasterize_size() (device,
  *                       256-byte aligned); keep it unchanged until the backward.
- *   pairs (host)        K. If K > capacity the image is incomplete and
- *                       GI_DEVERR_CAPACITY is raised, as with gi_bin_tiles.
+ *   pairs (host)        K. If K > capacity, GI_DEVERR_CAPACITY is raised, as
+ *                       with gi_bin_tiles, and nothing is rendered (out is
+ *                       left as it was).
  *   ws, ws_bytes        scratch of *backward_bytes.
- * The forward waits for its binning to learn K (not for the render behind
- * it) and so cannot be captured; the backward waits for nothing.
+ * The forward waits for its binning to learn K (not for the render, which it
+ * starts then) and so cannot be captured; the backward waits for nothing.
  * ---------------------------------------------------------------------- */
 GI_API gi_status gi_rasterize_size(int32_t n, gi_image img, int64_t capacity, size_t* forward_bytes,
                                    size_t* backward_bytes);

@@ -201,9 +201,9 @@ class GIRender(torch.autograd.Function):
     """Differentiable render: forward runs formation, binning and Eq. 7;
     backward recomputes the weights per tile (no per-pixel state saved).
     Each is one library call on buffers carved from one allocation (one host
-    synchronisation in the forward, for the pair count, while the render
-    already runs). A pair count above the first guess repeats the pass once
-    with the exact capacity."""
+    synchronisation in the forward, for the pair count; the render starts
+    behind it). A pair count above the first guess repeats formation and
+    binning once with the exact capacity."""
 
     @staticmethod
     def forward(ctx, means, chol, color, W: int, H: int, tile: int = 16):

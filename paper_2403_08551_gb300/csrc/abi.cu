@@ -448,11 +448,13 @@ gi_status gi_rasterize_forward(const float* means, const float* chol, const floa
     cudaError_t e = enqueue_form_bin(means, chol, color, single(img, n), capacity, b, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(w->k, b.k_dev, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaEventRecord(w->ev, s);
-    if (e == cudaSuccess) e = enqueue_plain_render(single(img, 0), b, out, s);
     if (e == cudaSuccess) e = cudaEventSynchronize(w->ev);
     if (e != cudaSuccess) return set_cuda_error(e, "gi_rasterize_forward");
     *pairs = *w->k;
-    return GI_OK;
+    // Behind the count: a list cut off at a short capacity is not worth
+    // rendering (the caller repeats the pass).
+    if (*pairs <= capacity) e = enqueue_plain_render(single(img, 0), b, out, s);
+    return e == cudaSuccess ? GI_OK : set_cuda_error(e, "gi_rasterize_forward");
 }
 
 gi_status gi_rasterize_backward(const void* state, size_t state_bytes, const float* chol, int32_t n, gi_image img,
