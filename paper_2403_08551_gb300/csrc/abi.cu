@@ -8,6 +8,7 @@
 #include <utility>
 
 #include "kernels.cuh"
+#include "pairs_wait.cuh"
 
 namespace gi {
 
@@ -105,41 +106,6 @@ cudaError_t enqueue_form_bin(const float* means, const float* chol, const float*
 cudaError_t enqueue_plain_render(const Batch& B, const RasterBufs& b, float* out, cudaStream_t s) {
     return launch_render(b.rec_binned, b.ranges, B, nullptr, out, nullptr, nullptr, nullptr, nullptr, device_status(),
                          s);
-}
-
-// The pinned word and event a host thread waits for a pair count with: one of
-// each per thread, for the device it last used, given back when it ends.
-struct PairsWait {
-    int dev = -1;
-    int64_t* k = nullptr;
-    cudaEvent_t ev = nullptr;
-    void drop() {
-        if (ev) cudaEventDestroy(ev);
-        if (k) cudaFreeHost(k);
-        ev = nullptr;
-        k = nullptr;
-        dev = -1;
-    }
-    ~PairsWait() { drop(); }  // after the runtime has shut down both calls only return an error
-};
-
-PairsWait* pairs_wait() {
-    thread_local PairsWait w;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-    if (w.dev != dev) {
-        w.drop();
-        void* p = nullptr;
-        if (cudaHostAlloc(&p, sizeof(int64_t), cudaHostAllocDefault) != cudaSuccess) return nullptr;
-        w.k = static_cast<int64_t*>(p);
-        if (cudaEventCreateWithFlags(&w.ev, cudaEventDisableTiming) != cudaSuccess) {
-            w.ev = nullptr;
-            w.drop();
-            return nullptr;
-        }
-        w.dev = dev;
-    }
-    return &w;
 }
 
 #define GI_REQUIRE(cond, ...)                                   \
