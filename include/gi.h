@@ -193,16 +193,27 @@ GI_API gi_status gi_render_pass(const float* means, const float* chol, const flo
 /* ------------------------------------------------------------------------
  * gi_rasterize_forward / gi_rasterize_backward -- the differentiable render
  * of an autograd program: gi_render_pass, then gi_render_backward of the same
- * pass, with everything the backward needs kept in one caller-owned buffer.
- *   state, state_bytes  *forward_bytes of gi_rasterize_size() (device,
+ * pass. What the backward reads is kept in one caller-owned buffer (40 bytes a
+ * pair of capacity); the rest of the forward's buffers is scratch that the
+ * caller may reuse as soon as the forward's work on the stream is done.
+ *   state, state_bytes  *state_bytes of gi_rasterize_split_size() (device,
  *                       256-byte aligned); keep it unchanged until the backward.
+ *   scratch, scratch_bytes  *scratch_bytes (device, 256-byte aligned).
  *   pairs (host)        K. If K > capacity, GI_DEVERR_CAPACITY is raised, as
  *                       with gi_bin_tiles, and nothing is rendered (out is
  *                       left as it was).
- *   ws, ws_bytes        scratch of *backward_bytes.
+ *   ws, ws_bytes        the backward's scratch of *backward_bytes.
+ * gi_rasterize_forward takes both buffers as one of *forward_bytes
+ * (gi_rasterize_size), which the backward accepts as its state.
  * The forward waits for its binning to learn K (not for the render, which it
  * starts then) and so cannot be captured; the backward waits for nothing.
  * ---------------------------------------------------------------------- */
+GI_API gi_status gi_rasterize_split_size(int32_t n, gi_image img, int64_t capacity, size_t* state_bytes,
+                                         size_t* scratch_bytes, size_t* backward_bytes);
+GI_API gi_status gi_rasterize_forward_split(const float* means, const float* chol, const float* color, int32_t n,
+                                            gi_image img, int64_t capacity, void* state, size_t state_bytes,
+                                            void* scratch, size_t scratch_bytes, float* out, int64_t* pairs,
+                                            gi_stream stream);
 GI_API gi_status gi_rasterize_size(int32_t n, gi_image img, int64_t capacity, size_t* forward_bytes,
                                    size_t* backward_bytes);
 GI_API gi_status gi_rasterize_forward(const float* means, const float* chol, const float* color, int32_t n,

@@ -42,6 +42,8 @@ SIGNATURES = {
     "gi_bin_tiles_noalloc": (i32, [P, P, P, i32, None, i64, P, P, P, P, P, P, P]),
     "gi_render": (i32, [P, P, None, P, P, P, P, P]),
     "gi_render_pass": (i32, [P, P, P, i32, None, i64, P, size_t, P, P, P, P, P, P, P, P, P, P, P]),
+    "gi_rasterize_split_size": (i32, [i32, None, i64, P, P, P]),
+    "gi_rasterize_forward_split": (i32, [P, P, P, i32, None, i64, P, size_t, P, size_t, P, P, P]),
     "gi_rasterize_size": (i32, [i32, None, i64, P, P]),
     "gi_rasterize_forward": (i32, [P, P, P, i32, None, i64, P, size_t, P, P, P]),
     "gi_rasterize_backward": (i32, [P, size_t, P, i32, None, i64, P, P, size_t, P, P, P, P]),

@@ -200,10 +200,11 @@ def codec_decode(stream: dict):
 class GIRender(torch.autograd.Function):
     """Differentiable render: forward runs formation, binning and Eq. 7;
     backward recomputes the weights per tile (no per-pixel state saved).
-    Each is one library call on buffers carved from one allocation (one host
-    synchronisation in the forward, for the pair count; the render starts
-    behind it). A pair count above the first guess repeats formation and
-    binning once with the exact capacity."""
+    Each is one library call (one host synchronisation in the forward, for
+    the pair count; the render starts behind it). What the backward reads
+    stays in one allocation, the forward's scratch is released on return. A
+    pair count above the first guess repeats formation and binning once with
+    the exact capacity."""
 
     @staticmethod
     def forward(ctx, means, chol, color, W: int, H: int, tile: int = 16):
@@ -214,21 +215,25 @@ class GIRender(torch.autograd.Function):
         n = means.shape[0]
         img = _img(W, H, tile)
         stream = L.stream_handle()
-        fwd, bwd, pairs = ctypes.c_size_t(0), ctypes.c_size_t(0), ctypes.c_int64(0)
+        fwd, tmp, bwd, pairs = ctypes.c_size_t(0), ctypes.c_size_t(0), ctypes.c_size_t(0), ctypes.c_int64(0)
         cap = max(4096, 8 * n)
         out = None
         for _ in range(2):
-            L.check(lib.gi_rasterize_size(n, img, cap, ctypes.byref(fwd), ctypes.byref(bwd)), "gi_rasterize_size")
+            L.check(lib.gi_rasterize_split_size(n, img, cap, ctypes.byref(fwd), ctypes.byref(tmp), ctypes.byref(bwd)),
+                    "gi_rasterize_split_size")
             state = torch.empty((fwd.value,), dtype=torch.uint8, device=means.device)
+            scratch = torch.empty((tmp.value,), dtype=torch.uint8, device=means.device)
             if out is None:
                 out = torch.empty((H, W, 3), dtype=torch.float32, device=means.device)
-            L.check(lib.gi_rasterize_forward(L.ptr(means) if n else None, L.ptr(chol) if n else None,
-                                             L.ptr(color) if n else None, n, img, cap, L.ptr(state), fwd.value,
-                                             L.ptr(out), ctypes.byref(pairs), stream), "gi_rasterize_forward")
+            L.check(lib.gi_rasterize_forward_split(L.ptr(means) if n else None, L.ptr(chol) if n else None,
+                                                   L.ptr(color) if n else None, n, img, cap, L.ptr(state), fwd.value,
+                                                   L.ptr(scratch), tmp.value, L.ptr(out), ctypes.byref(pairs), stream),
+                    "gi_rasterize_forward")
             if pairs.value <= cap:
                 break
             device_errors(clear=True)  # drop the capacity bit raised by the short guess
             cap = pairs.value
+            del state, scratch
         else:
             raise L.GIError("gi_rasterize_forward: capacity retry failed")
         ctx.save_for_backward(chol.detach())

@@ -61,30 +61,40 @@ size_t raster_dl_bytes(const gi_image& img) {
     return up256((size_t)single(img, 0).total_tiles * img.tile * img.tile * 12);
 }
 
-// Carve-up of gi_rasterize_forward's state; bytes = its size.
-RasterBufs raster_layout(void* base, int32_t n, const gi_image& img, int64_t capacity, size_t& bytes) {
+struct RasterBytes {
+    size_t state, scratch, backward;
+};
+
+// Carve-up of a differentiable pass: in `state` what its backward reads, in
+// `scratch` what the forward needs besides.
+RasterBufs raster_layout(void* state, void* scratch, int32_t n, const gi_image& img, int64_t capacity,
+                         RasterBytes& bytes) {
     RasterBufs b{};
     const int tiles = single(img, n).total_tiles;
-    b.ws = bin_ws_layout(base, n, capacity, tiles);
     const size_t N = (size_t)(n > 0 ? n : 1), cap = (size_t)capacity;
-    char* p = static_cast<char*>(base);
-    size_t off = up256(b.ws.bytes);
+    char* p = static_cast<char*>(state);
+    size_t off = 0;
     auto take = [&](size_t x) -> void* {
         const size_t o = off;
         off += up256(x);
         return p ? p + o : nullptr;
     };
-    b.rec = static_cast<float4*>(take(N * 32));
-    b.rect = static_cast<int4*>(take(N * 16));
-    b.cnt = static_cast<int32_t*>(take(N * 4));
-    b.keys = static_cast<uint32_t*>(take(cap * 4));
-    b.ids = static_cast<uint32_t*>(take(cap * 4));
-    b.ranges = static_cast<int2*>(take((size_t)tiles * 8));
     b.rec_binned = static_cast<float4*>(take(cap * 32));
+    b.keys = static_cast<uint32_t*>(take(cap * 4));
     b.emit = static_cast<uint32_t*>(take(cap * 4));
+    b.cnt = static_cast<int32_t*>(take(N * 4));
     b.pair_off = static_cast<int64_t*>(take((N + 1) * 8));
     b.k_dev = static_cast<int64_t*>(take(8));
-    bytes = off;
+    bytes.state = off;
+    b.ws = bin_ws_layout(scratch, n, capacity, tiles);
+    p = static_cast<char*>(scratch);
+    off = up256(b.ws.bytes);
+    b.rec = static_cast<float4*>(take(N * 32));
+    b.rect = static_cast<int4*>(take(N * 16));
+    b.ids = static_cast<uint32_t*>(take(cap * 4));
+    b.ranges = static_cast<int2*>(take((size_t)tiles * 8));
+    bytes.scratch = off;
+    bytes.backward = raster_partial_bytes(capacity) + raster_dl_bytes(img);
     return b;
 }
 
@@ -374,35 +384,52 @@ gi_status gi_render_pass(const float* means, const float* chol, const float* col
     return GI_OK;
 }
 
-gi_status gi_rasterize_size(int32_t n, gi_image img, int64_t capacity, size_t* forward_bytes, size_t* backward_bytes) {
-    gi_status st = check_image(img, "gi_rasterize_size");
+gi_status gi_rasterize_split_size(int32_t n, gi_image img, int64_t capacity, size_t* state_bytes,
+                                  size_t* scratch_bytes, size_t* backward_bytes) {
+    gi_status st = check_image(img, "gi_rasterize_split_size");
     if (st != GI_OK) return st;
-    GI_REQUIRE(forward_bytes && backward_bytes, "gi_rasterize_size: NULL pointer");
+    GI_REQUIRE(state_bytes && scratch_bytes && backward_bytes, "gi_rasterize_split_size: NULL pointer");
     GI_REQUIRE(n >= 0 && capacity >= 1 && capacity <= kMaxCapacity,
-               "gi_rasterize_size: bad n (%d) or capacity (%lld)", n, (long long)capacity);
-    size_t bytes = 0;
-    raster_layout(nullptr, n, img, capacity, bytes);
-    *forward_bytes = bytes;
-    *backward_bytes = raster_partial_bytes(capacity) + raster_dl_bytes(img);
+               "gi_rasterize_split_size: bad n (%d) or capacity (%lld)", n, (long long)capacity);
+    RasterBytes bytes{};
+    raster_layout(nullptr, nullptr, n, img, capacity, bytes);
+    *state_bytes = bytes.state;
+    *scratch_bytes = bytes.scratch;
+    *backward_bytes = bytes.backward;
     return GI_OK;
 }
 
-gi_status gi_rasterize_forward(const float* means, const float* chol, const float* color, int32_t n, gi_image img,
-                               int64_t capacity, void* state, size_t state_bytes, float* out, int64_t* pairs,
-                               gi_stream stream) {
-    NvtxRange nvtx_("gi_rasterize_forward");
-    size_t need = 0, unused = 0;
-    gi_status st = gi_rasterize_size(n, img, capacity, &need, &unused);
+gi_status gi_rasterize_size(int32_t n, gi_image img, int64_t capacity, size_t* forward_bytes, size_t* backward_bytes) {
+    GI_REQUIRE(forward_bytes && backward_bytes, "gi_rasterize_size: NULL pointer");
+    size_t state = 0, scratch = 0, backward = 0;
+    gi_status st = gi_rasterize_split_size(n, img, capacity, &state, &scratch, &backward);
     if (st != GI_OK) return st;
-    GI_REQUIRE(state && out && pairs && (n == 0 || (means && chol && color)), "gi_rasterize_forward: NULL pointer");
-    GI_REQUIRE(aligned(state, 256) && aligned(means, 4) && aligned(chol, 4) && aligned(color, 4) && aligned(out, 4),
+    *forward_bytes = state + scratch;
+    *backward_bytes = backward;
+    return GI_OK;
+}
+
+gi_status gi_rasterize_forward_split(const float* means, const float* chol, const float* color, int32_t n,
+                                     gi_image img, int64_t capacity, void* state, size_t state_bytes, void* scratch,
+                                     size_t scratch_bytes, float* out, int64_t* pairs, gi_stream stream) {
+    NvtxRange nvtx_("gi_rasterize_forward");
+    size_t need_state = 0, need_scratch = 0, unused = 0;
+    gi_status st = gi_rasterize_split_size(n, img, capacity, &need_state, &need_scratch, &unused);
+    if (st != GI_OK) return st;
+    GI_REQUIRE(state && scratch && out && pairs && (n == 0 || (means && chol && color)),
+               "gi_rasterize_forward: NULL pointer");
+    GI_REQUIRE(aligned(state, 256) && aligned(scratch, 256) && aligned(means, 4) && aligned(chol, 4) &&
+                   aligned(color, 4) && aligned(out, 4),
                "gi_rasterize_forward: misaligned pointer");
-    GI_REQUIRE(state_bytes >= need, "gi_rasterize_forward: state %zu bytes < %zu needed", state_bytes, need);
-    const RasterBufs b = raster_layout(state, n, img, capacity, need);
+    GI_REQUIRE(state_bytes >= need_state && scratch_bytes >= need_scratch,
+               "gi_rasterize_forward: state %zu or scratch %zu bytes < %zu, %zu needed", state_bytes, scratch_bytes,
+               need_state, need_scratch);
+    RasterBytes bytes{};
+    const RasterBufs b = raster_layout(state, scratch, n, img, capacity, bytes);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     *pairs = 0;
     if (n == 0) {
-        st = gi_bin_tiles(nullptr, nullptr, nullptr, 0, img, capacity, state, b.ws.bytes, b.keys, b.ids,
+        st = gi_bin_tiles(nullptr, nullptr, nullptr, 0, img, capacity, scratch, b.ws.bytes, b.keys, b.ids,
                           reinterpret_cast<int32_t*>(b.ranges), reinterpret_cast<float*>(b.rec_binned), b.pair_off,
                           b.k_dev, stream);
         return st == GI_OK ? gi_render(reinterpret_cast<float*>(b.rec_binned), reinterpret_cast<int32_t*>(b.ranges),
@@ -423,19 +450,32 @@ gi_status gi_rasterize_forward(const float* means, const float* chol, const floa
     return e == cudaSuccess ? GI_OK : set_cuda_error(e, "gi_rasterize_forward");
 }
 
+gi_status gi_rasterize_forward(const float* means, const float* chol, const float* color, int32_t n, gi_image img,
+                               int64_t capacity, void* state, size_t state_bytes, float* out, int64_t* pairs,
+                               gi_stream stream) {
+    size_t need = 0, scratch = 0, unused = 0;
+    gi_status st = gi_rasterize_split_size(n, img, capacity, &need, &scratch, &unused);
+    if (st != GI_OK) return st;
+    GI_REQUIRE(state_bytes >= need + scratch, "gi_rasterize_forward: state %zu bytes < %zu needed", state_bytes,
+               need + scratch);
+    return gi_rasterize_forward_split(means, chol, color, n, img, capacity, state, need,
+                                      state ? static_cast<char*>(state) + need : nullptr, scratch, out, pairs, stream);
+}
+
 gi_status gi_rasterize_backward(const void* state, size_t state_bytes, const float* chol, int32_t n, gi_image img,
                                 int64_t capacity, const float* dl_dout, void* ws, size_t ws_bytes, float* g_means,
                                 float* g_chol, float* g_color, gi_stream stream) {
     NvtxRange nvtx_("gi_rasterize_backward");
-    size_t fwd = 0, bwd = 0;
-    gi_status st = gi_rasterize_size(n, img, capacity, &fwd, &bwd);
+    size_t need = 0, unused = 0, bwd = 0;
+    gi_status st = gi_rasterize_split_size(n, img, capacity, &need, &unused, &bwd);
     if (st != GI_OK) return st;
     if (n == 0) return GI_OK;
     GI_REQUIRE(state && chol && dl_dout && ws && g_means && g_chol && g_color, "gi_rasterize_backward: NULL pointer");
     GI_REQUIRE(aligned(state, 256) && aligned(ws, 256), "gi_rasterize_backward: misaligned pointer");
-    GI_REQUIRE(state_bytes >= fwd && ws_bytes >= bwd, "gi_rasterize_backward: state %zu or workspace %zu bytes < %zu, %zu",
-               state_bytes, ws_bytes, fwd, bwd);
-    const RasterBufs b = raster_layout(const_cast<void*>(state), n, img, capacity, fwd);
+    GI_REQUIRE(state_bytes >= need && ws_bytes >= bwd, "gi_rasterize_backward: state %zu or workspace %zu bytes < %zu, %zu",
+               state_bytes, ws_bytes, need, bwd);
+    RasterBytes bytes{};
+    const RasterBufs b = raster_layout(const_cast<void*>(state), nullptr, n, img, capacity, bytes);
     const Batch B = single(img, n);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     float4* partial = static_cast<float4*>(ws);
