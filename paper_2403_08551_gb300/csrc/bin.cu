@@ -680,33 +680,15 @@ __device__ __forceinline__ void sort_block(int blk, int K, SortSmem& sm, const u
     }
 }
 
-// Keys per thread for K keys. A block is latency-bound (ranking key by key,
-// barriers, look-back) and fills an SM's registers, so the sort takes as long as
-// its waves of kSortWave blocks: the fewest keys a thread that need one wave,
-// beyond that 12 if that needs no more waves than 16. Measured with 512 threads
-// at 16 / 12 / 8 / 4 keys (256 x 16 before): render of 1,000 x 1,422 / 51,000
-// Gaussians 67 / - / 59 / 56 us (65), 2040x1356 / 100,000 85 / - / 79.5 / 80.4
-// (90.7), 1,738 x 1,506 / 130,000 98 / 94.5 / 101 / 101 (104), 1,827 x 1,396 /
-// 200,000 124 / - / 130 / 132 (130); step of 1,633 x 1,443 / 104,000 at tile 8 316
-// / 310.5; 24 keys gain 5 us more there and cost 1 us everywhere else (spills).
-__device__ __forceinline__ int sort_items(int K) {
-    constexpr int w = kSortWave * kSortThreads;  // keys of one wave per item
-    if (K <= 4 * w) return 4;
-    if (K <= 8 * w) return 8;
-    if (K <= 12 * w) return 12;
-    if (K <= 16 * w) return 16;
-    return (K + 12 * w - 1) / (12 * w) > (K + 16 * w - 1) / (16 * w) ? 16 : 12;
-}
-
 __global__ void __launch_bounds__(kSortThreads, 1) k_onesweep(
     const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
-    uint32_t* __restrict__ vals_out, const int64_t* __restrict__ k_dev, int64_t capacity, int shift, int dbits,
-    const uint32_t* __restrict__ hist, uint32_t* __restrict__ lookback, uint32_t* __restrict__ ticket,
+    uint32_t* __restrict__ vals_out, const int64_t* __restrict__ k_dev, int64_t capacity, int wave, int shift,
+    int dbits, const uint32_t* __restrict__ hist, uint32_t* __restrict__ lookback, uint32_t* __restrict__ ticket,
     uint32_t* __restrict__ status) {
     __shared__ SortSmem sm;
     pdl_wait();
     const int K = (int)min(*k_dev, capacity);
-    const int items = sort_items(K);
+    const int items = sort_items(K, wave);
     // the blocks past the last key: out before they take a ticket
     if ((int64_t)blockIdx.x * kSortThreads * items >= K) return;
     if (threadIdx.x == 0) sm.s_ticket = atomicAdd(ticket, 1u);
@@ -795,14 +777,6 @@ __global__ void k_ranges(const uint32_t* __restrict__ keys, uint32_t* __restrict
     }
 }
 
-// Blocks that a sort of up to `capacity` keys may use (sort_items: never more
-// than the waves that 16 keys a thread take).
-int64_t sort_blocks(int64_t capacity) {
-    auto blocks = [&](int items) { return (capacity + kSortThreads * items - 1) / (kSortThreads * items); };
-    const int64_t wave16 = int64_t(kSortWave) * kSortThreads * 16;
-    return std::max<int64_t>(1, std::min<int64_t>(blocks(4), kSortWave * ((capacity + wave16 - 1) / wave16)));
-}
-
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
@@ -818,7 +792,8 @@ RadixPlan radix_plan(int total_tiles) {
 BinWs bin_ws_layout(void* base, int64_t n, int64_t capacity, int total_tiles, bool with_owner) {
     const RadixPlan rp = radix_plan(total_tiles);
     const int64_t nblk = std::max<int64_t>(1, (n + kProjBlock - 1) / kProjBlock);
-    const int64_t sblk = sort_blocks(capacity);
+    const int wave = sm_count();
+    const int64_t sblk = sort_blocks(capacity, wave);
     const int chunk = cm_chunk(n);
     const int64_t nchunks = std::max<int64_t>(1, (n + chunk - 1) / chunk);
     const int64_t cap = std::max<int64_t>(1, capacity);
@@ -832,6 +807,8 @@ BinWs bin_ws_layout(void* base, int64_t n, int64_t capacity, int total_tiles, bo
     BinWs w{};
     w.cm_path = cm_applies(n, total_tiles);
     w.chunk = chunk;
+    w.sort_wave = wave;
+    w.sort_grid = (int)sblk;
     w.blk_sum = static_cast<int64_t*>(take(nblk * sizeof(int64_t)));
     if (w.cm_path) {
         w.cm = static_cast<uint32_t*>(take((size_t)nchunks * total_tiles * 4));
@@ -874,7 +851,6 @@ cudaError_t launch_bin(const int4* rect, const int32_t* cnt, const float4* rec, 
     const RadixPlan rp = radix_plan(B.total_tiles);
     const int n = B.total_gauss;
     const int nblk = std::max(1, (n + kProjBlock - 1) / kProjBlock);
-    const int64_t sblk = sort_blocks(capacity);
     if (!blk_sum_ready) {
         ZeroJob zj{};
         zj.p[0] = ws.zero;
@@ -895,11 +871,10 @@ cudaError_t launch_bin(const int4* rect, const int32_t* cnt, const float4* rec, 
     e = smem_optin(reinterpret_cast<const void*>(k_onesweep), kSortStageBytes);
     if (e != cudaSuccess) return e;
     for (int ps = 0; ps < rp.passes; ++ps) {
-        e = launch_pdl(k_onesweep, dim3((unsigned)sblk), dim3(kSortThreads), (size_t)kSortStageBytes, s, ka, va, kb,
-                       vb, k_dev, capacity,
-                       ps * rp.dbits, rp.dbits, ws.hist + ps * kHistReplicas * kMaxRadix,
-                       ws.lookback + (size_t)ps * sblk * kMaxRadix,
-                       ws.tickets + ps, status);
+        e = launch_pdl(k_onesweep, dim3((unsigned)ws.sort_grid), dim3(kSortThreads), (size_t)kSortStageBytes, s, ka, va,
+                       kb, vb, k_dev, capacity, ws.sort_wave, ps * rp.dbits, rp.dbits,
+                       ws.hist + ps * kHistReplicas * kMaxRadix,
+                       ws.lookback + (size_t)ps * ws.sort_grid * kMaxRadix, ws.tickets + ps, status);
         if (e != cudaSuccess) return e;
         std::swap(ka, kb);
         std::swap(va, vb);

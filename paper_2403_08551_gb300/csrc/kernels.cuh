@@ -2,6 +2,7 @@
 // fit context (fit.cu). Not part of the public ABI.
 #pragma once
 #include "common.cuh"
+#include "sort_plan.cuh"
 
 namespace gi {
 
@@ -32,13 +33,11 @@ struct RadixPlan {
 RadixPlan radix_plan(int total_tiles);
 
 constexpr int kProjBlock = 256;        // Gaussians per projection / emit block
-constexpr int kSortThreads = 512;      // threads per onesweep block
-constexpr int kSortWave = 152;         // onesweep blocks that run at the same time (one per SM)
 constexpr int kMaxDigitBits = 9;       // radix digits of at most 9 bits (512 buckets)
 constexpr int kMaxRadix = 1 << kMaxDigitBits;
 constexpr int kMaxPasses = 4;          // 31-bit keys at most
 constexpr int kHistReplicas = 8;       // copies of each pass's digit histogram (spread the emit's atomics)
-constexpr int kSortStageBytes = kSortThreads * 16 * 8;  // keys + values of a block staged in digit order
+constexpr int kSortStageBytes = kSortThreads * kSortMaxItems * 8;  // keys + values of a block staged in digit order
 
 // Count-matrix binning (bin_cm.cu): chunks of cm_chunk(n) Gaussians; used when
 // the batch has at most kCmMaxTiles tiles and 128-Gaussian rows x tiles <=
@@ -52,7 +51,7 @@ bool cm_applies(int64_t n, int total_tiles);
 
 // Binning workspace carve-up. [zero, zero + zero_words) holds every buffer
 // that must be zero before a binning pass. Radix path: keys_tmp, vals_tmp,
-// hist [passes][kHistReplicas][kMaxRadix], lookback [passes][sort_blocks][kMaxRadix]. Count-matrix path: cm
+// hist [passes][kHistReplicas][kMaxRadix], lookback [passes][sort_grid][kMaxRadix]. Count-matrix path: cm
 // [chunks][tiles], chunk_sum [chunks], tile_tot [tiles] (column totals).
 struct BinWs {
     bool cm_path;
@@ -70,6 +69,8 @@ struct BinWs {
     uint32_t* hist;       // [passes][kHistReplicas][kMaxRadix] (radix)
     uint64_t* blk_lb;     // [ceil(n / kProjBlock)] published block prefixes of the key emission (radix)
     uint32_t* lookback;
+    int sort_wave;        // onesweep blocks that run at the same time: the device's SMs (radix)
+    int sort_grid;        // onesweep blocks launched, sort_blocks(capacity, sort_wave) (radix)
     uint32_t* tickets;    // [4]
     size_t bytes;
 };
