@@ -515,7 +515,6 @@ struct SortSmem {
     uint32_t s_base[kMaxRadix];   // global position of the block's first key of each digit
     uint32_t s_boff[kMaxRadix];   // block-local position of the first key of each digit
     uint32_t s_warp[32];
-    uint32_t s_tot0;
     uint32_t s_ticket;
 };
 
@@ -526,7 +525,7 @@ __device__ __forceinline__ void sort_block(int blk, int K, SortSmem& sm, const u
                                            const uint32_t* __restrict__ hist, uint32_t* __restrict__ lookback,
                                            uint32_t* __restrict__ status) {
     constexpr int NW = kSortThreads / 32;
-    constexpr int DPT = kMaxRadix / kSortThreads;  // digits per thread in the per-digit phases
+    static_assert(kSortThreads == kMaxRadix, "one digit per thread in the per-digit phases");
     extern __shared__ uint32_t s_stage[];          // keys, then values, in digit order
     constexpr int kTile = kSortThreads * ITEMS;
     const int64_t start = (int64_t)blk * kTile;
@@ -570,54 +569,31 @@ __device__ __forceinline__ void sort_block(int blk, int K, SortSmem& sm, const u
     }
     __syncthreads();
 
-    // Per digit: exclusive offsets of the warps, the block's total, published
-    // at once (an inclusive prefix for the first block).
-    uint32_t tot[DPT];
+    // Per digit d = threadIdx.x: exclusive offsets of the warps, the block's
+    // total, published at once (an inclusive prefix for the first block).
+    const int d = threadIdx.x;
+    uint32_t tot = 0;
+    if (d < radix) {
 #pragma unroll
-    for (int q = 0; q < DPT; ++q) {
-        const int d = threadIdx.x + q * kSortThreads;
-        tot[q] = 0;
-        if (d < radix) {
-#pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                const uint32_t v = sm.s_wc[w][d];
-                sm.s_wc[w][d] = tot[q];
-                tot[q] += v;
-            }
-            st_relaxed_u32(lookback + (size_t)blk * kMaxRadix + d, (blk == 0 ? kFlagPre : kFlagAgg) | tot[q]);
+        for (int w = 0; w < NW; ++w) {
+            const uint32_t v = sm.s_wc[w][d];
+            sm.s_wc[w][d] = tot;
+            tot += v;
         }
+        st_relaxed_u32(lookback + (size_t)blk * kMaxRadix + d, (blk == 0 ? kFlagPre : kFlagAgg) | tot);
     }
-    // Global digit bases: exclusive scan of this pass's histogram, digits
-    // [0, kSortThreads) then [kSortThreads, kMaxRadix).
-    uint32_t hex[DPT];
-    {
-        uint32_t carry = 0, lcarry = 0;
+    // Global digit base: exclusive scan of this pass's histogram.
+    uint32_t h = 0;
+    if (d < radix) {
 #pragma unroll
-        for (int q = 0; q < DPT; ++q) {
-            const int d = threadIdx.x + q * kSortThreads;
-            uint32_t h = 0;
-            if (d < radix) {
-#pragma unroll
-                for (int rep = 0; rep < kHistReplicas; ++rep) h += hist[rep * kMaxRadix + d];
-            }
-            const uint32_t incl = block_incl_scan<uint32_t>(h, sm.s_warp);  // ends with a barrier
-            hex[q] = carry + incl - h;
-            if (threadIdx.x == kSortThreads - 1) sm.s_tot0 = incl;
-            __syncthreads();
-            carry += sm.s_tot0;
-            __syncthreads();
-            const uint32_t lincl = block_incl_scan<uint32_t>(tot[q], sm.s_warp);
-            if (d < radix) sm.s_boff[d] = lcarry + lincl - tot[q];
-            if (threadIdx.x == kSortThreads - 1) sm.s_tot0 = lincl;
-            __syncthreads();
-            lcarry += sm.s_tot0;
-            __syncthreads();
-        }
+        for (int rep = 0; rep < kHistReplicas; ++rep) h += hist[rep * kMaxRadix + d];
     }
-#pragma unroll
-    for (int q = 0; q < DPT; ++q) {
-        const int d = threadIdx.x + q * kSortThreads;
-        if (d >= radix) continue;
+    // (the local scan first: after the histogram's, which waits for its loads, a
+    // render of 2040x1356 / 100,000 takes 84.0 us instead of 83.2)
+    const uint32_t lex = block_incl_scan<uint32_t>(tot, sm.s_warp) - tot;  // its barriers also publish s_wc
+    if (d < radix) sm.s_boff[d] = lex;
+    const uint32_t hex = block_incl_scan<uint32_t>(h, sm.s_warp) - h;  // and these s_boff
+    if (d < radix) {
         uint32_t excl = 0;
         if (blk > 0) {
             // Windowed look-back: kWin predecessor words loaded at once
@@ -650,9 +626,9 @@ __device__ __forceinline__ void sort_block(int blk, int K, SortSmem& sm, const u
                     if (spins > 16) __nanosleep(64);
                 }
             }
-            st_relaxed_u32(lookback + (size_t)blk * kMaxRadix + d, kFlagPre | ((excl + tot[q]) & kValMask));
+            st_relaxed_u32(lookback + (size_t)blk * kMaxRadix + d, kFlagPre | ((excl + tot) & kValMask));
         }
-        sm.s_base[d] = hex[q] + excl;
+        sm.s_base[d] = hex + excl;
     }
     // Stage the block's keys in digit order, then write each digit's run
     // with consecutive threads (coalesced stores).
