@@ -97,12 +97,13 @@ __device__ __forceinline__ float opacity_of(float t) {
     return ok && t >= kSigmoidMin ? o : (float)sigmoid_fp64((double)t);
 }
 
-// size * sigmoid(2 x), rounded once (size = 0 .. 2^31 - 1, split into two floats).
+// size * sigmoid(2 x), rounded once (size = 0 .. 2^31 - 1, split into two
+// floats, the first rounded towards zero so that it is a whole number in range).
 __device__ __forceinline__ float raw_position(float x, int size) {
     const float t = __fmul_rn(2.f, x);
     float hi, lo;
     sigmoid_dd(t, hi, lo);
-    const float sh = (float)size, sl = (float)(size - (int)sh);
+    const float sh = __int2float_rz(size), sl = (float)(size - (int)sh);
     const float m = __fmul_rn(hi, sh);
     bool ok;
     const float p = round_once(m, __fmaf_rn(lo, sh, __fmaf_rn(hi, sl, __fmaf_rn(hi, sh, -m))), ok);

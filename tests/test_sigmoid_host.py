@@ -1,7 +1,8 @@
 """The formation's double-float sigmoid (csrc/sigmoid.cuh) compiled for the host,
 every operation with its single rounding, against long double: the relative
 error of the pair from the threshold up, and opacities and App. C.1 positions
-equal to size * sigmoid rounded once over the whole range. (The formula (tanh x + 1) / 2, which FP64 loses digits in for
+equal to size * sigmoid rounded once over the whole range, sizes that no float
+holds among them. (The formula (tanh x + 1) / 2, which FP64 loses digits in for
 negative x, is no reference below x = -4.)"""
 import os
 import shutil
@@ -27,6 +28,7 @@ static float __fmaf_rn(float a, float b, float c) { return std::fma(a, b, c); }
 static float __frcp_rn(float a) { return 1.0f / a; }
 static double __dmul_rn(double a, double b) { return a * b; }
 static int __float2int_rn(float a) { return (int)std::nearbyint(a); }
+static float __int2float_rz(int a) { float f = (float)a; return (double)f > (double)a ? std::nextafter(f, 0.0f) : f; }
 static float __int_as_float(int a) { float f; std::memcpy(&f, &a, 4); return f; }
 using std::fabs; using std::fmin; using std::rint;
 #include "sigmoid.cuh"
@@ -55,7 +57,7 @@ int main() {
             bad += opacity_of(t) != (float)ref(t);
         }
     if (bad) std::printf("%ld opacities\\n", bad);
-    for (int size : {1, 517, 2040, 65535, 16777217}) {
+    for (int size : {1, 517, 2040, 65535, 16777217, 2147483585, 2147483647}) {
         bad = 0;
         for (float hi : {1.f, 4.f, 12.f, 45.f})
             for (int i = 0; i < 100000; ++i) {
@@ -77,6 +79,8 @@ int main() {
 def test_error_and_rounding(tmp_path):
     (tmp_path / "main.cpp").write_text(MAIN)
     exe = tmp_path / "main"
-    subprocess.run(["g++", "-std=c++17", "-O1", "-ffp-contract=off", "-x", "c++", "-I", CSRC, str(tmp_path / "main.cpp"),
+    subprocess.run(["g++", "-std=c++17", "-O1", "-ffp-contract=off",
+                    "-fsanitize=float-cast-overflow,signed-integer-overflow", "-fsanitize-undefined-trap-on-error",
+                    "-x", "c++", "-I", CSRC, str(tmp_path / "main.cpp"),
                     "-o", str(exe)], check=True)
     assert subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout == ""
