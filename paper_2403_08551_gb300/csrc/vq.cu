@@ -17,12 +17,17 @@ namespace {
 // The FP64 sum of up to eight floats rounded to FP32, on the FP32 units (with
 // FP64 a three-stage decode took five times a two-stage one): s + e is the
 // running sum and the errors of its additions (Knuth, TAOCP 2, 4.2.2), p the sum
-// of the magnitudes, q the smallest but for zeros. If q >= 2^-22 p, all terms are
-// multiples of 2^-45 p: then e (below 2^-21 p) and the FP64 sum are both exact, so
-// that s + e rounds as it does. Otherwise (terms of very different size,
-// infinities, NaN) get() is false and the caller sums in FP64. Three stages,
-// 64 entries: 1 M Gaussians 88 -> 16.5 us, 3.2 M x 256 entries 256 -> 43.6 us (what
-// bounds it there is the codebook rows' bank conflicts).
+// of the magnitudes, q the smallest but for zeros. With u the last unit of q, every
+// term is a multiple of u and q < 2^24 u. If q >= 2^-22 p, then p < 2^46 u at every
+// addition, |s| <= p (rounding is monotone), and an addition's error is a multiple
+// of u of at most 2^21 u. The first addition is exact, so the seven others of eight
+// terms leave |e| <= 7 * 2^21 u < 2^24 u: e is exact in FP32 (for more terms it
+// need not be), the FP64 sum is exact below 2^53 u, and s + e rounds as it does.
+// Otherwise (terms of very different size, infinities, NaN) get() is false and the
+// caller sums in FP64. Three stages, 64 entries: 1 M Gaussians 88 -> 16.5 us, 3.2 M
+// x 256 entries 256 -> 43.6 us (what bounds it there is the codebook rows' bank
+// conflicts).
+constexpr int kRowSumTerms = 8;
 struct RowSum {
     float s = 0.f, e = 0.f, p = 0.f, q = 3.402823466e38f;
     __device__ __forceinline__ void add(float x) {
@@ -173,6 +178,7 @@ __device__ __forceinline__ void vq_quad(const uint32_t (&w)[MAXS], const float4*
 #pragma unroll
             for (int c = 0; c < 3; ++c) o[j][c] = f[c];
         } else {
+            static_assert(MAXS <= kRowSumTerms, "RowSum is exact for eight terms");
             RowSum sum[3];
 #pragma unroll
             for (int st = 0; st < MAXS; ++st) {
