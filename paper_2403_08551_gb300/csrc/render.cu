@@ -300,11 +300,15 @@ __device__ __forceinline__ void render_tile(int t, uint32_t& phase, const RSmem<
 // One block per tile, tiles in index order. The explicit minimum of one block
 // lets the compiler use the registers it wants (98 instead of 80 at split 4,
 // where shared memory bounds the residency anyway): render stage 85.7 -> 79.5
-// us at 2040x1356 / 200k with the wide partial stores below (87.7 before both),
-// 178 -> 172 us on 16 uneven images. Not at tile 32, whose blocks would take 68
-// registers instead of 48 and fewer would be resident: with a crowd of tiles in
-// one corner the step takes 304 to 342 us without the bound and 324 to 336 with
-// it, by where the corner lies (1120x1109 / 108k; 316 to 352 before both).
+// us at 2040x1356 / 200k with the wide partial stores above (87.7 before both),
+// 178 -> 172 us on 16 uneven images. Not at tile 32, where it takes 68 registers
+// instead of 48 and three blocks fit an SM instead of five. Over 60 steps of
+// random sizes (256x256 to 2040x1356, half with a crowd in one corner) that is
+// 3.3 % faster on average, up to 15 % on small crowded images, but a step of a
+// large crowded image, which the last tiles' blocks end, can lose: 1083x804 /
+// 104k 319 -> 337 us (325 before the wide stores), 1264x826 / 33k 150.8 -> 152.2.
+// Without the bound none of the 60 is slower than before the wide stores. 64
+// registers and four blocks: 2.9 % faster on average, 3.7 % slower at worst.
 template <class Cfg>
 __global__ void __launch_bounds__(Cfg::kThreads, Cfg::T == 32 ? 0 : 1) k_render(const float4* __restrict__ rec_binned,
                                                           const int2* __restrict__ ranges, Batch B,
