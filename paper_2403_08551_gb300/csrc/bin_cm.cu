@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kCmScanThreads) k_colscan(uint32_t* __restrict
 // [kTilesPerThread i, kTilesPerThread (i + 1)), one block scan) and adds it
 // to its chunk's row of P. Lane masks s_m[k][t] (bit l set when local
 // Gaussian 32 k + l covers tile t) are built with atomicOr, which is
-// order-independent; then pair (t, g), g = 128 b + 32 k + l, lands at
+// order-independent; then pair (t, g), g = CH b + 32 k + l, lands at
 //   start[t] + P[b][t] + sum_{k' < k} popc(s_m[k'][t]) + popc(s_m[k][t] & bits below l),
 // i.e. ascending g inside the tile; the block writes ids, records and
 // emission indices there. pair_off = exclusive scan of cnt in emission
