@@ -5,6 +5,7 @@ step of the rasterizer runs in libgi's kernels.
 from __future__ import annotations
 
 import ctypes
+import functools
 from dataclasses import dataclass
 from typing import List, Optional, Sequence
 
@@ -197,6 +198,18 @@ def codec_decode(stream: dict):
     return means, chol, color
 
 
+@functools.lru_cache(maxsize=256)
+def _raster_sizes(n: int, W: int, H: int, tile: int, cap: int, device: int):
+    """Bytes of a differentiable pass on the current device (number `device`:
+    the sort's scratch goes by its SM count): state, scratch, backward
+    scratch. Kept per shape: the library call takes 6 us of each pass, about
+    what the second allocation costs."""
+    state, scratch, backward = ctypes.c_size_t(0), ctypes.c_size_t(0), ctypes.c_size_t(0)
+    L.check(L.load().gi_rasterize_split_size(n, _img(W, H, tile), cap, ctypes.byref(state), ctypes.byref(scratch),
+                                             ctypes.byref(backward)), "gi_rasterize_split_size")
+    return state.value, scratch.value, backward.value
+
+
 class GIRender(torch.autograd.Function):
     """Differentiable render: forward runs formation, binning and Eq. 7;
     backward recomputes the weights per tile (no per-pixel state saved).
@@ -215,19 +228,18 @@ class GIRender(torch.autograd.Function):
         n = means.shape[0]
         img = _img(W, H, tile)
         stream = L.stream_handle()
-        fwd, tmp, bwd, pairs = ctypes.c_size_t(0), ctypes.c_size_t(0), ctypes.c_size_t(0), ctypes.c_int64(0)
+        pairs = ctypes.c_int64(0)
         cap = max(4096, 8 * n)
         out = None
         for _ in range(2):
-            L.check(lib.gi_rasterize_split_size(n, img, cap, ctypes.byref(fwd), ctypes.byref(tmp), ctypes.byref(bwd)),
-                    "gi_rasterize_split_size")
-            state = torch.empty((fwd.value,), dtype=torch.uint8, device=means.device)
-            scratch = torch.empty((tmp.value,), dtype=torch.uint8, device=means.device)
+            fwd, tmp, bwd = _raster_sizes(n, img.width, img.height, img.tile, cap, torch.cuda.current_device())
+            state = torch.empty((fwd,), dtype=torch.uint8, device=means.device)
+            scratch = torch.empty((tmp,), dtype=torch.uint8, device=means.device)
             if out is None:
                 out = torch.empty((H, W, 3), dtype=torch.float32, device=means.device)
             L.check(lib.gi_rasterize_forward_split(L.ptr(means) if n else None, L.ptr(chol) if n else None,
-                                                   L.ptr(color) if n else None, n, img, cap, L.ptr(state), fwd.value,
-                                                   L.ptr(scratch), tmp.value, L.ptr(out), ctypes.byref(pairs), stream),
+                                                   L.ptr(color) if n else None, n, img, cap, L.ptr(state), fwd,
+                                                   L.ptr(scratch), tmp, L.ptr(out), ctypes.byref(pairs), stream),
                     "gi_rasterize_forward")
             if pairs.value <= cap:
                 break
@@ -238,7 +250,7 @@ class GIRender(torch.autograd.Function):
             raise L.GIError("gi_rasterize_forward: capacity retry failed")
         ctx.save_for_backward(chol.detach())
         ctx.state = state
-        ctx.meta = (n, img, cap, fwd.value, bwd.value)
+        ctx.meta = (n, img, cap, fwd, bwd)
         return out
 
     @staticmethod
